@@ -254,6 +254,31 @@ struct StepArgs {
   SymArgs sym;               // the symmetric kernel's plan and buffers
 };
 
+// ---- the team kernel (few running events) --------------------------------
+// One CTA's part in an event's steps: rank of `size` CTAs of the slot's team.
+struct TeamEntry {
+  int32_t slot, rank, size, pad;
+};
+constexpr int kTeamCtaThreads = 512;
+constexpr int kTeamRow = 4;             // own carriers per row of pair work
+constexpr int kTeamSmem = 220 * 1024;   // dynamic shared memory of a CTA at most
+// Source chunks of an event with `its` iterations of 64 sources: at most
+// eight, of at least four iterations (all but the last of equal length).
+__host__ __device__ inline int team_chunks(int its) {
+  if (its <= 4) return 1;
+  const int most = (its + 3) / 4 < 8 ? (its + 3) / 4 : 8;
+  const int len = (its + most - 1) / most;
+  return (its + len - 1) / len;
+}
+// Shared memory of a CTA in a team of `size` for an event of n_h + n_e
+// carriers: every position (padded to 64 per species) and the partial sums
+// of its tasks.
+__host__ __device__ inline int64_t team_smem_bytes(int64_t n_h, int64_t n_e, int64_t size) {
+  const int64_t its = (n_h + 63) / 64 + (n_e + 63) / 64;
+  const int64_t rows = (n_h + kTeamRow - 1) / kTeamRow + (n_e + kTeamRow - 1) / kTeamRow;
+  return 12 * 64 * its + 12 * kTeamRow * ((rows + size - 1) / size) * team_chunks((int)its);
+}
+
 // ---- kernel launchers (cts_kernels.cu) ----------------------------------
 struct Variant {
   int nt;       // threads per CTA
@@ -271,6 +296,12 @@ size_t variant_smem(int v);
 // Steps k0 .. k0 + nk - 1 of the chunk in one launch (nk > 1 needs a dynamic
 // variant and a slot-major plan).
 cudaError_t launch_step(int v, const StepArgs& a, int k0, int nk, int grid, cudaStream_t s);
+// The team kernel over CTAs [0, grid), a cooperative launch (all CTAs
+// resident); team_prepare raises its shared-memory limit on the current device
+// (at sim_init).
+cudaError_t team_prepare();
+cudaError_t launch_team(const StepArgs& a, const TeamEntry* ctas, int k0, int nk, int grid,
+                        size_t smem, cudaStream_t s);
 cudaError_t launch_update(const StepArgs& a, int k, int n_slots_list, const int32_t* slot_list,
                           int grid, cudaStream_t s);
 cudaError_t launch_init(const Phys& ph, Arena A, SlotDev* slots, const int32_t* slot_list,

@@ -416,15 +416,70 @@ __device__ __noinline__ void window_potentials(double x, double y, double z, dou
   }
 }
 
-// Position update of one active carrier (Eqs. 3, 5, 6; Sec. 2.1) at arena
-// index idx, carrier id and state st, position (x, y, z) at the start of the
-// step, with the field E (V/um) of its step: collection/exit and (SHADOW) the
-// next shadow entry.  When the induced charge is recorded, returns H times
-// the charge (units of e) the move induces on the collecting surface
-// (Shockley-Ramo, weighting potential 1 - z/H, the end point held on [0, H]);
-// else 0.  IND: 0 records nothing, 1 the whole surface, 2 also adds
-// q (phi(end) - phi(start)) of the 3 x 3 window's pixels to qpx.  *retired
-// (when given) is set when the carrier left.
+// Move of one active carrier in one step (Eqs. 3, 5, 6; Sec. 2.1) from
+// (x, y, z) with the pair field E (V/um) and the step's diffusion normals n:
+// the new position, whether the displacement is finite, and the state the
+// carrier leaves with (kStateActive: it stays).
+__device__ __forceinline__ int move_carrier(const Phys& ph, int spec, float3 n, float Ex, float Ey,
+                                            float Ez, double& x, double& y, double& z,
+                                            bool& finite) {
+  if (ph.drift) Ez -= drift_E(ph, (float)z);
+  const float Em = sqrtf(Ex * Ex + Ey * Ey + Ez * Ez);
+  const float mu = mobility_f(ph, spec, Em);
+  const float c = (spec ? -mu : mu) * ph.f_dt;
+  float dx = c * Ex, dy = c * Ey, dz = c * Ez;
+  if (ph.diffusion) {
+    const float amp = sqrtf(2.0f * mu * ph.f_kT * ph.f_dt);
+    dx = fmaf(amp, n.x, dx);
+    dy = fmaf(amp, n.y, dy);
+    dz = fmaf(amp, n.z, dz);
+  }
+  finite = isfinite(dx) && isfinite(dy) && isfinite(dz);
+  x += (double)dx;
+  y += (double)dy;
+  z += (double)dz;
+  int retire = kStateActive;
+  if (spec == 0) {
+    if (z <= 0.0) retire = kStateCollected;
+    else if (z > ph.H) z = 2.0 * ph.H - z;
+  } else {
+    if (z >= ph.H) retire = kStateExited;
+    else if (z < 0.0) z = -z;
+  }
+  return retire;
+}
+
+// H times the charge (units of e) that a move from (x0, y0, z0) to (x, y, z)
+// induces on the collecting surface (Shockley-Ramo, weighting potential
+// 1 - z/H, the end point held on [0, H]), or 0 when it is not recorded.
+// IND 1: the whole surface; 2 also adds q (phi(end) - phi(start)) of the
+// 3 x 3 window's pixels to qpx.
+template <int IND>
+__device__ __forceinline__ double induced_charge(const StepArgs& a, int spec, double x0, double y0,
+                                                 double z0, double x, double y, double z,
+                                                 double* qpx) {
+  const Phys& ph = a.ph;
+  if (IND == 1 && !a.induced) return 0.0;
+  const double zb = fmin(fmax(z, 0.0), ph.H);
+  if constexpr (IND == 2) {
+    float w0[9], w1[9];
+    window_potentials(x0, y0, z0, ph.wp_x0, ph.wp_y0, ph.pitch, ph.grid_n, ph.H, ph.wp_pairs,
+                      ph.wp_c3, ph.wp_c5, w0);
+    window_potentials(x, y, zb, ph.wp_x0, ph.wp_y0, ph.pitch, ph.grid_n, ph.H, ph.wp_pairs,
+                      ph.wp_c3, ph.wp_c5, w1);
+#pragma unroll
+    for (int j = 0; j < 9; ++j)
+      qpx[j] += spec ? (double)w0[j] - (double)w1[j] : (double)w1[j] - (double)w0[j];
+  }
+  if (!a.induced) return 0.0;
+  return spec ? zb - z0 : z0 - zb;
+}
+
+// Position update of one active carrier at arena index idx, carrier id and
+// state st, position (x, y, z) at the start of the step, with the field E
+// (V/um) of its step: collection/exit and (SHADOW) the next shadow entry.
+// Returns the induced charge (IND > 0; see induced_charge).  *retired (when
+// given) is set when the carrier left.
 template <int IND, bool SHADOW = true>
 __device__ __forceinline__ double update_carrier_at(const StepArgs& a, SlotDev* S, int slot,
                                                   int spec, int64_t idx, int id, int8_t st,
@@ -443,30 +498,12 @@ __device__ __forceinline__ double update_carrier_at(const StepArgs& a, SlotDev* 
   }
 #endif
   [[maybe_unused]] const double x_start = x, y_start = y, z_start = z;
-  if (ph.drift) Ez -= drift_E(ph, (float)z);
-  const float Em = sqrtf(Ex * Ex + Ey * Ey + Ez * Ez);
-  const float mu = mobility_f(ph, spec, Em);
-  const float c = (spec ? -mu : mu) * ph.f_dt;
-  float dx = c * Ex, dy = c * Ey, dz = c * Ez;
-  if (ph.diffusion) {
-    const float3 n = normals_f(stream_words(S->seed, S->event_id, 0u, (uint32_t)id, (uint32_t)step));
-    const float amp = sqrtf(2.0f * mu * ph.f_kT * ph.f_dt);
-    dx = fmaf(amp, n.x, dx);
-    dy = fmaf(amp, n.y, dy);
-    dz = fmaf(amp, n.z, dz);
-  }
-  if (!(isfinite(dx) && isfinite(dy) && isfinite(dz))) atomicOr(&S->flags, kErrNumeric);
-  x += (double)dx;
-  y += (double)dy;
-  z += (double)dz;
-  int retire = 0;
-  if (spec == 0) {
-    if (z <= 0.0) retire = kStateCollected;
-    else if (z > ph.H) z = 2.0 * ph.H - z;
-  } else {
-    if (z >= ph.H) retire = kStateExited;
-    else if (z < 0.0) z = -z;
-  }
+  float3 n = make_float3(0.0f, 0.0f, 0.0f);
+  if (ph.diffusion)
+    n = normals_f(stream_words(S->seed, S->event_id, 0u, (uint32_t)id, (uint32_t)step));
+  bool finite;
+  const int retire = move_carrier(ph, spec, n, Ex, Ey, Ez, x, y, z, finite);
+  if (!finite) atomicOr(&S->flags, kErrNumeric);
   a.A.px[idx] = x;
   a.A.py[idx] = y;
   a.A.pz[idx] = z;
@@ -483,24 +520,10 @@ __device__ __forceinline__ double update_carrier_at(const StepArgs& a, SlotDev* 
   } else if constexpr (SHADOW) {
     shout[idx] = make_float4((float)(x - S->ax), (float)(y - S->ay), (float)(z - azn), 0.0f);
   }
-  if constexpr (IND == 0) {
+  if constexpr (IND == 0)
     return 0.0;
-  } else {
-    if (IND == 1 && !a.induced) return 0.0;
-    const double zb = fmin(fmax(z, 0.0), ph.H);
-    if constexpr (IND == 2) {
-      float w0[9], w1[9];
-      window_potentials(x_start, y_start, z_start, ph.wp_x0, ph.wp_y0, ph.pitch, ph.grid_n, ph.H,
-                        ph.wp_pairs, ph.wp_c3, ph.wp_c5, w0);
-      window_potentials(x, y, zb, ph.wp_x0, ph.wp_y0, ph.pitch, ph.grid_n, ph.H, ph.wp_pairs,
-                        ph.wp_c3, ph.wp_c5, w1);
-#pragma unroll
-      for (int j = 0; j < 9; ++j)
-        qpx[j] += spec ? (double)w0[j] - (double)w1[j] : (double)w1[j] - (double)w0[j];
-    }
-    if (!a.induced) return 0.0;
-    return spec ? zb - z_start : z_start - zb;
-  }
+  else
+    return induced_charge<IND>(a, spec, x_start, y_start, z_start, x, y, z, qpx);
 }
 
 // update_carrier_at for the carrier at arena index idx, its id, state and
@@ -1560,6 +1583,434 @@ __global__ void __launch_bounds__(NT, 1) sym_kernel(StepArgs a, int k0, int nk) 
   }
 }
 
+// ---------------------------------------------------------------------------
+// The team kernel: the steps of a chunk when few events run.
+// ---------------------------------------------------------------------------
+// With few resident events a step is bound by latency, not by the FP32 pipe:
+// the queue kernels above spend 20-50 us per step on pulling units, splitting
+// tiles, combining the pieces and publishing a step's completion.  Here each
+// running event gets a team of CTAs (in proportion to its pair work; one CTA
+// per SM, all resident at once: a cooperative launch) for all steps of the
+// chunk.  Every CTA keeps the FP32 positions of the whole event in shared
+// memory and computes the field of its own carriers (a contiguous range)
+// from all of them, so no partial field leaves the CTA, and the own carriers'
+// FP64 positions stay with the thread that updates them.
+//
+// What a step exchanges is the new FP32 positions, through the arena's
+// shadow: entry w of a position written for step s holds s as an integer, so
+// a reader waits on the data itself (16-byte single-copy atomic accesses, no
+// counter, no fence, one L2 round trip).  A step's entry cannot be taken for
+// another's: an event's steps only increase, init_kernel and the other step
+// kernels write w = 0.  Two buffers are enough: a CTA writes step s + 1 after
+// it has read every entry of step s, and an entry of step s is written after
+// its CTA has read all of step s - 1, whose buffer step s + 1 reuses.
+//
+// Work inside a CTA: a task is a row of kTeamR own carriers against one of the
+// event's source chunks (team_chunks: at most eight, a few iterations of 64
+// sources each, two per lane).  A warp reduces a task's sums over its lanes (a
+// fixed tree) into shared memory and the updating thread adds its row's chunks
+// in order.  Rows and chunks follow from the event alone, so a carrier's field
+// has the same bits whatever the size of the team and whatever else runs.
+// Four helper warps first draw the first 128 own carriers' diffusion normals
+// and the next frame anchors; they take pair tasks too when there are enough.
+constexpr int kTeamR = 4;           // own carriers per row
+constexpr int kTeamPairWarps = 12;
+constexpr int kTeamHelp = 128;      // helper threads
+constexpr int kTeamThreads = 32 * kTeamPairWarps + kTeamHelp;
+constexpr int kTeamFewTasks = 48;   // up to this many tasks: helpers take none
+static_assert(kTeamThreads == kTeamCtaThreads && kTeamR == kTeamRow, "host planning constants");
+
+__device__ __forceinline__ float4 ld_entry(const float4* p) {
+  unsigned long long lo, hi;
+  asm volatile(
+      "{\n .reg .b128 t;\n ld.relaxed.gpu.global.b128 t, [%2];\n mov.b128 {%0, %1}, t;\n}\n"
+      : "=l"(lo), "=l"(hi)
+      : "l"(p)
+      : "memory");
+  return make_float4(__uint_as_float((uint32_t)lo), __uint_as_float((uint32_t)(lo >> 32)),
+                     __uint_as_float((uint32_t)hi), __uint_as_float((uint32_t)(hi >> 32)));
+}
+__device__ __forceinline__ void st_entry(float4* p, float x, float y, float z, int tag) {
+  const unsigned long long lo =
+      (unsigned long long)__float_as_uint(x) | ((unsigned long long)__float_as_uint(y) << 32);
+  const unsigned long long hi =
+      (unsigned long long)__float_as_uint(z) | ((unsigned long long)(uint32_t)tag << 32);
+  asm volatile(
+      "{\n .reg .b128 t;\n mov.b128 t, {%1, %2};\n st.relaxed.gpu.global.b128 [%0], t;\n}\n" ::"l"(
+          p),
+      "l"(lo), "l"(hi)
+      : "memory");
+}
+
+// acc_r += d w over iterations [it0, it1) of 64 sources from x[], y[], z[]
+// (float2 per lane and iteration), d = r_i - r_j, or r_j - r_i (NEG).
+template <bool NEG>
+__device__ __forceinline__ void team_pairs(const float* __restrict__ xs,
+                                           const float* __restrict__ ys,
+                                           const float* __restrict__ zs, int lane, int it0,
+                                           int it1, const float (&xi)[kTeamR],
+                                           const float (&yi)[kTeamR], const float (&zi)[kTeamR],
+                                           float2 (&ax)[kTeamR], float2 (&ay)[kTeamR],
+                                           float2 (&az)[kTeamR], float eps2s) {
+  const float2 m1 = make_float2(-1.0f, -1.0f);
+  const float2 eps2 = make_float2(eps2s, eps2s);
+  float2 x2[kTeamR], y2[kTeamR], z2[kTeamR];
+#pragma unroll
+  for (int r = 0; r < kTeamR; ++r) {
+    x2[r] = make_float2(xi[r], xi[r]);
+    y2[r] = make_float2(yi[r], yi[r]);
+    z2[r] = make_float2(zi[r], zi[r]);
+  }
+#pragma unroll 2
+  for (int it = it0; it < it1; ++it) {
+    const int j = 64 * it + 2 * lane;
+    const float2 qx = *reinterpret_cast<const float2*>(xs + j);
+    const float2 qy = *reinterpret_cast<const float2*>(ys + j);
+    const float2 qz = *reinterpret_cast<const float2*>(zs + j);
+#pragma unroll
+    for (int r = 0; r < kTeamR; ++r) {
+      const float2 dx = NEG ? __ffma2_rn(x2[r], m1, qx) : __ffma2_rn(qx, m1, x2[r]);
+      const float2 dy = NEG ? __ffma2_rn(y2[r], m1, qy) : __ffma2_rn(qy, m1, y2[r]);
+      const float2 dz = NEG ? __ffma2_rn(z2[r], m1, qz) : __ffma2_rn(qz, m1, z2[r]);
+      float2 r2 = __ffma2_rn(dz, dz, eps2);
+      r2 = __ffma2_rn(dy, dy, r2);
+      r2 = __ffma2_rn(dx, dx, r2);
+      const float2 rs = make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+      const float2 w = __fmul2_rn(__fmul2_rn(rs, rs), rs);
+      ax[r] = __ffma2_rn(dx, w, ax[r]);
+      ay[r] = __ffma2_rn(dy, w, ay[r]);
+      az[r] = __ffma2_rn(dz, w, az[r]);
+    }
+  }
+}
+
+// Sums the four rows' three components over the warp's lanes (a fixed tree);
+// lane l with l mod 8 == 0 ends with carrier l / 8's sums in v[0..2].
+__device__ __forceinline__ void team_reduce(float (&v)[3 * kTeamR], int lane) {
+  static_assert(kTeamR == 4, "two halving exchanges");
+  const bool h16 = lane & 16, h8 = lane & 8;
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    const float give = h16 ? v[q] : v[q + 6], keep = h16 ? v[q + 6] : v[q];
+    v[q] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const float give = h8 ? v[q] : v[q + 3], keep = h8 ? v[q + 3] : v[q];
+    v[q] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+  }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+    for (int q = 0; q < 3; ++q) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+}
+
+// CTA b runs its part ctas[b] of one event's steps k0 .. k0 + nk - 1.
+template <int IND>
+__global__ void __launch_bounds__(kTeamThreads, 1) team_kernel(StepArgs a, const TeamEntry* ctas,
+                                                               int k0, int nk) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ int s_count[2][2];      // [step parity][species]: active carriers
+  __shared__ double s_azn[2];        // the next step's frame anchors
+  __shared__ float s_off[2];         // [step parity]: electron frame minus hole frame
+  // event constants and the helper threads' own carriers (each touched by its
+  // own thread only), here rather than in registers: the pair loop needs those
+  __shared__ uint64_t s_seed, s_event;
+  __shared__ int64_t s_base, s_ebase;
+  __shared__ double s_ax, s_ay;
+  __shared__ double s_x[kTeamHelp], s_y[kTeamHelp], s_z[kTeamHelp];
+  __shared__ int s_id[kTeamHelp];    // carrier id; -1: padding or retired
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const TeamEntry T = ctas[blockIdx.x];
+  SlotDev* S = a.slots + T.slot;
+  const Phys& ph = a.ph;
+#ifdef CTS_BOUNDS_CHECK
+  if (T.slot < 0 || T.slot >= a.S || T.size < 1 || T.rank < 0 || T.rank >= T.size || k0 < 0 ||
+      k0 + nk > kMaxK || !slot_in_arena(a.A, S) || S->n_h > S->cap_h || S->n_e > S->cap_e ||
+      team_smem_bytes(S->n_h, S->n_e, T.size) > kTeamSmem) {
+    if (tid == 0) atomicOr(a.err, kErrBounds);
+    return;
+  }
+#endif
+  if (!S->running) return;
+  const int nh = S->n_h, ne = S->n_e, n = nh + ne;
+  const int step0 = S->step0;
+  const int ih = (nh + 63) >> 6, ie = (ne + 63) >> 6, its = ih + ie, NP = its << 6;
+  float* xs = reinterpret_cast<float*>(smem_raw);
+  float* ys = xs + NP;
+  float* zs = ys + NP;
+  float* part = zs + NP;  // [rows][chunks][3 * kTeamR]
+  // rows of the event: the holes', then the electrons'; this CTA's range
+  const int gh = (nh + kTeamR - 1) / kTeamR, gt = gh + (ne + kTeamR - 1) / kTeamR;
+  const int g0 = (int)((int64_t)gt * T.rank / T.size), g1 = (int)((int64_t)gt * (T.rank + 1) / T.size);
+  const int nch = team_chunks(its), chunk = (its + nch - 1) / nch;
+  const int rows = g1 - g0, tasks = rows * nch;
+  const int own = kTeamR * rows;
+  // own carrier c: its species, index in the species range (-1: padding)
+  auto locate = [&](int c, int& spec) {
+    const int g = g0 + c / kTeamR;
+    spec = g >= gh;
+    const int i = kTeamR * (spec ? g - gh : g) + c % kTeamR;
+    return i < (spec ? ne : nh) ? i : -1;
+  };
+  // the padding of the two position segments stays parked
+  for (int j = nh + tid; j < 64 * ih; j += kTeamThreads) xs[j] = ys[j] = zs[j] = kParked;
+  for (int j = 64 * ih + ne + tid; j < NP; j += kTeamThreads) xs[j] = ys[j] = zs[j] = kParked;
+  // a helper thread's own carrier lives in its registers; the other threads'
+  // carriers in the arena
+  const bool help = warp >= kTeamPairWarps;
+  const int hc = tid - 32 * kTeamPairWarps;
+  double azc = 0.0;  // helper lanes 0 and 1: their species' frame anchor
+  if (help) {
+    const int64_t base = S->base, ebase = base + S->cap_h;
+    int hspec = 0, hi = -1, keep = -1;
+    if (hc < own) hi = locate(hc, hspec);
+    if (hi >= 0) {
+      const int64_t hidx = (hspec ? ebase : base) + hi;
+      int hid = a.A.cid[hidx];
+#ifdef CTS_BOUNDS_CHECK
+      if (hid < 0 || hid >= S->n_total) {
+        atomicOr(a.err, kErrBounds);
+        hid = 0;
+      }
+#endif
+      if ((a.A.cstate[base + hid] & kStateMask) == kStateActive) keep = hid;
+      s_x[hc] = a.A.px[hidx];
+      s_y[hc] = a.A.py[hidx];
+      s_z[hc] = a.A.pz[hidx];
+    }
+    s_id[hc] = keep;
+    if (hc < 2) azc = S->az[step0 + k0 & 1][hc];
+    if (hc == 0) {
+      s_count[0][0] = s_count[0][1] = s_count[1][0] = s_count[1][1] = 0;
+      s_off[step0 + k0 & 1] = (float)(S->az[step0 + k0 & 1][1] - azc);
+      s_seed = S->seed;
+      s_event = S->event_id;
+      s_base = base;
+      s_ebase = ebase;
+      s_ax = S->ax;
+      s_ay = S->ay;
+    }
+  }
+  __syncthreads();
+  for (int kq = 0; kq < nk; ++kq) {
+    const int k = k0 + kq, step = step0 + k, p = step & 1;
+    // 1. the event's positions of this step into shared memory; counts of
+    // the active carriers on the way
+    bool ok = true;
+    {
+      int ch = 0, ce = 0;
+      const float4* shh = a.A.sh[p] + s_base;
+      const float4* she = a.A.sh[p] + s_ebase - nh;
+      constexpr int kBatch = 5;
+      for (int e0 = tid; e0 < n; e0 += kBatch * kTeamThreads) {
+        float4 q[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+          const int e = e0 + u * kTeamThreads;
+          if (e < n) q[u] = ld_entry((e < nh ? shh : she) + e);
+        }
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+          const int e = e0 + u * kTeamThreads;
+          if (e < n) {
+            if (kq > 0 && __float_as_int(q[u].w) != step) {
+              // not written yet: bounded wait (about two seconds)
+              const unsigned long long t0 = sym_now();
+              do {
+                q[u] = ld_entry((e < nh ? shh : she) + e);
+                if (__float_as_int(q[u].w) == step) break;
+                if (sym_now() - t0 > kCountWaitNs) ok = false;
+              } while (ok);
+            }
+            const bool act = q[u].x < 0.5f * kParked;
+            const int j = e < nh ? e : 64 * ih + (e - nh);
+            xs[j] = q[u].x;
+            ys[j] = q[u].y;
+            zs[j] = q[u].z;
+            if (e < nh) ch += act;
+            else ce += act;
+          }
+        }
+      }
+      ch = __reduce_add_sync(0xffffffffu, ch);
+      ce = __reduce_add_sync(0xffffffffu, ce);
+      if (lane == 0) {
+        if (ch) atomicAdd(&s_count[p][0], ch);
+        if (ce) atomicAdd(&s_count[p][1], ce);
+      }
+    }
+    if (__syncthreads_or(!ok)) {
+      if (tid == 0) atomicOr(a.err, kErrTimeout);
+      return;
+    }
+    const int nah = s_count[p][0], nae = s_count[p][1];
+    if (nah <= 0 || (int64_t)step >= ph.max_steps) break;
+    // 2. the pair field of the own carriers
+    float3 hn = make_float3(0.0f, 0.0f, 0.0f);
+    if (help) {
+      if (hc < 32) {
+        double azn = azc;
+        if (hc < 2) azn = anchor_next(ph, hc, azc);
+        const double other = __shfl_down_sync(0xffffffffu, azn, 1);
+        if (hc < 2) s_azn[hc] = azn;
+        if (hc == 0) {
+          s_off[p ^ 1] = (float)(other - azn);
+          s_count[p ^ 1][0] = s_count[p ^ 1][1] = 0;
+          if (T.rank == 0) slot_duties(a, S, step, p, nah, nae, azn, other);
+        }
+        azc = azn;
+      }
+      if (ph.diffusion && s_id[hc] >= 0)
+        hn = normals_f(stream_words(s_seed, s_event, 0u, (uint32_t)s_id[hc], (uint32_t)step));
+    }
+    const int workers = tasks > kTeamFewTasks ? kTeamPairWarps + kTeamHelp / 32 : kTeamPairWarps;
+    if (ph.repulsion && warp < workers) {
+      const float off = s_off[p];
+      const int q1 = (int)((int64_t)tasks * (warp + 1) / workers);
+      for (int q = (int)((int64_t)tasks * warp / workers); q < q1; ++q) {
+        const int row = q / nch, it0 = (q - row * nch) * chunk, it1 = min(its, it0 + chunk);
+        const int g = g0 + row;
+        const int spec = g >= gh;
+        const int si = spec ? 64 * ih + kTeamR * (g - gh) : kTeamR * g;
+        const float4 X = *reinterpret_cast<const float4*>(xs + si);
+        const float4 Y = *reinterpret_cast<const float4*>(ys + si);
+        const float4 Z = *reinterpret_cast<const float4*>(zs + si);
+        const float xi[kTeamR] = {X.x, X.y, X.z, X.w}, yi[kTeamR] = {Y.x, Y.y, Y.z, Y.w};
+        float2 ax[kTeamR], ay[kTeamR], az[kTeamR];
+#pragma unroll
+        for (int r = 0; r < kTeamR; ++r) ax[r] = ay[r] = az[r] = make_float2(0.0f, 0.0f);
+        if (it0 < ih) {  // hole sources, in the hole frame
+          const float o = spec ? off : 0.0f;
+          const float zi[kTeamR] = {Z.x + o, Z.y + o, Z.z + o, Z.w + o};
+          team_pairs<false>(xs, ys, zs, lane, it0, min(it1, ih), xi, yi, zi, ax, ay, az, ph.f_eps2);
+        }
+        if (it1 > ih) {  // electron sources, in the electron frame
+          const float o = spec ? 0.0f : off;
+          const float zi[kTeamR] = {Z.x - o, Z.y - o, Z.z - o, Z.w - o};
+          team_pairs<true>(xs, ys, zs, lane, max(it0, ih), it1, xi, yi, zi, ax, ay, az, ph.f_eps2);
+        }
+        float v[3 * kTeamR];
+#pragma unroll
+        for (int r = 0; r < kTeamR; ++r) {
+          v[3 * r] = ax[r].x + ax[r].y;
+          v[3 * r + 1] = ay[r].x + ay[r].y;
+          v[3 * r + 2] = az[r].x + az[r].y;
+        }
+        team_reduce(v, lane);
+        if ((lane & 7) == 0) {
+          float* dst = part + q * (3 * kTeamR) + 3 * (lane >> 3);
+          dst[0] = v[0];
+          dst[1] = v[1];
+          dst[2] = v[2];
+        }
+      }
+    }
+    __syncthreads();
+    // 3. update of the own carriers and their entries for the next step
+    auto field = [&](int c, float& Ex, float& Ey, float& Ez) {
+      Ex = Ey = Ez = 0.0f;
+      if (!ph.repulsion) return;
+      const float* src = part + (c / kTeamR) * nch * (3 * kTeamR) + 3 * (c % kTeamR);
+      for (int q = 0; q < nch; ++q, src += 3 * kTeamR) {
+        Ex += src[0];
+        Ey += src[1];
+        Ez += src[2];
+      }
+      Ex *= ph.f_kc;
+      Ey *= ph.f_kc;
+      Ez *= ph.f_kc;
+    };
+    [[maybe_unused]] double qi = 0.0;
+    [[maybe_unused]] double qpx[9] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    // the carrier's move; false once it has left
+    auto advance = [&](int spec, int64_t idx, int id, float3 nrm, int c, double& x, double& y,
+                       double& z) {
+      float Ex, Ey, Ez;
+      field(c, Ex, Ey, Ez);
+      [[maybe_unused]] const double x0 = x, y0 = y, z0 = z;
+      bool finite;
+      const int retire = move_carrier(ph, spec, nrm, Ex, Ey, Ez, x, y, z, finite);
+      const bool stay = retire == kStateActive;
+      st_entry(a.A.sh[p ^ 1] + idx, stay ? (float)(x - s_ax) : kParked,
+               stay ? (float)(y - s_ay) : kParked,
+               stay ? (float)(z - s_azn[spec]) : kParked, step + 1);
+      if (!finite) atomicOr(&S->flags, kErrNumeric);
+      if (!stay) {
+        const int64_t rid = s_base + id;
+        a.A.cstate[rid] = (int8_t)((spec ? kElectronBit : 0) | retire);
+        a.A.rstep[rid] = step;
+        if (retire == kStateCollected) {
+          a.A.fx[rid] = x;
+          a.A.fy[rid] = y;
+        }
+        atomicAdd(&a.ret[((int64_t)k * a.S + T.slot) * 2 + spec], 1);
+      }
+      if constexpr (IND > 0) qi += induced_charge<IND>(a, spec, x0, y0, z0, x, y, z, qpx);
+      return stay;
+    };
+    if (help) {
+      int spec;
+      const int i = hc < own ? locate(hc, spec) : -1;
+      if (i >= 0) {
+        const int64_t idx = (spec ? s_ebase : s_base) + i;
+        const int id = s_id[hc];
+        if (id < 0) {
+          st_entry(a.A.sh[p ^ 1] + idx, kParked, kParked, kParked, step + 1);
+        } else {
+          double x = s_x[hc], y = s_y[hc], z = s_z[hc];
+          if (!advance(spec, idx, id, hn, hc, x, y, z)) s_id[hc] = -1;
+          s_x[hc] = x;
+          s_y[hc] = y;
+          s_z[hc] = z;
+        }
+      }
+    } else {
+      for (int c = kTeamHelp + tid; c < own; c += 32 * kTeamPairWarps) {
+        int spec;
+        const int i = locate(c, spec);
+        if (i < 0) continue;
+        const int64_t idx = (spec ? s_ebase : s_base) + i;
+        int id = a.A.cid[idx];
+#ifdef CTS_BOUNDS_CHECK
+        if (id < 0 || id >= S->n_total) {
+          atomicOr(a.err, kErrBounds);
+          id = 0;
+        }
+#endif
+        if ((a.A.cstate[s_base + id] & kStateMask) != kStateActive) {
+          st_entry(a.A.sh[p ^ 1] + idx, kParked, kParked, kParked, step + 1);
+          continue;
+        }
+        float3 nrm = make_float3(0.0f, 0.0f, 0.0f);
+        if (ph.diffusion)
+          nrm = normals_f(stream_words(s_seed, s_event, 0u, (uint32_t)id, (uint32_t)step));
+        double x = a.A.px[idx], y = a.A.py[idx], z = a.A.pz[idx];
+        advance(spec, idx, id, nrm, c, x, y, z);
+        a.A.px[idx] = x;
+        a.A.py[idx] = y;
+        a.A.pz[idx] = z;
+      }
+    }
+    if constexpr (IND > 0) {
+      __syncwarp();
+      add_induced(a, k, T.slot, qi);
+      if constexpr (IND == 2) add_induced_px(a, k, T.slot, qpx);
+    }
+  }
+  if (help && hc < own) {
+    int spec;
+    const int i = locate(hc, spec);
+    if (i >= 0) {
+      const int64_t idx = (spec ? s_ebase : s_base) + i;
+      a.A.px[idx] = s_x[hc];
+      a.A.py[idx] = s_y[hc];
+      a.A.pz[idx] = s_z[hc];
+    }
+  }
+}
+
+
 // Update alone: reads the field written by a FIELD_ONLY step launch.
 // PX: the instantiation that records the 3 x 3 window's pixels too.
 template <bool PX>
@@ -1817,6 +2268,7 @@ __global__ void __launch_bounds__(kAuxThreads) init_kernel(Phys ph, Arena A, Slo
     } else {
       A.sh[0][idx] = make_float4((float)(x - ax0), (float)(y - ay0), (float)(z - az0), 0.0f);
     }
+    A.sh[1][idx] = make_float4(kParked, kParked, kParked, 0.0f);  // no step's entry yet
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -2600,6 +3052,32 @@ cudaError_t launch_step(int v, const StepArgs& a, int k0, int nk, int grid, cuda
   (a.induced_px ? e.fn_px : (a.induced ? e.fn_ind : e.fn))<<<grid, e.nt, smem_of(e), s>>>(
       a, k0, nk);
   return cudaGetLastError();
+}
+
+cudaError_t team_prepare() {
+  for (auto* fn : {team_kernel<0>, team_kernel<1>, team_kernel<2>}) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kTeamSmem);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t launch_team(const StepArgs& a, const TeamEntry* ctas, int k0, int nk, int grid,
+                        size_t smem, cudaStream_t s) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.gridDim = dim3((unsigned)grid, 1, 1);
+  cfg.blockDim = dim3(kTeamThreads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, a.induced_px ? team_kernel<2> : a.induced ? team_kernel<1>
+                                                                            : team_kernel<0>,
+                            a, ctas, k0, nk);
 }
 
 cudaError_t launch_update(const StepArgs& a, int k, int n_slots_list, const int32_t* slot_list,

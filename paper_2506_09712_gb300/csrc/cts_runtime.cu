@@ -59,6 +59,24 @@ constexpr int kSymVariantLarge = 12;  // sym_nt256_r8_warp
 constexpr int kSymLargeTiles = 640;
 constexpr int kPairVariant = 1;  // nt256_r2_jpair_dyn
 constexpr int kSymVariantPlain = 0;  // sym_nt384_r8_warp
+// The team kernel takes a chunk while the running events' carrier pairs are
+// below kTeamMaxLoad times the largest event's carriers.  Below, a step is
+// bound by latency, which grows with the event in the per-pair kernel; above,
+// by the pair loop, where the per-pair kernel is the faster one (2.8e12 against
+// 2.2e12 pairs/s).  Microseconds per step, team / per-pair kernel: 829 carriers,
+// 1 / 8 / 32 / 64 events 4.8 / 18.2, 7.2 / 18.7, 19.8 / 21.2, 35.4 / 30.1; 2210
+// carriers, 1 / 8 / 16 events 7.5 / 25.1, 24.0 / 28.8, 45.6 / 41.5; 5525
+// carriers, 1 / 2 / 4 / 8 events 19.7 / 51.0, 33.4 / 50.6, 59.5 / 58.3,
+// 111.5 / 96.4; 8000 carriers, 1 / 4 events 27.3 / 59.0, 83.5 / 96.2: the two
+// meet at 2.1e4 to 3.1e4.  SERVE keeps the queue kernels: a cooperative launch
+// waits until all its SMs are free at once, which would put a stream of
+// requests behind whatever else its process runs on the GPU (and the events of
+// a stream are meant to overlap: alone, an 8 keV event of a served stream
+// takes 8.7 ms with teams, 26 ms without).
+constexpr double kTeamMaxLoad = 2.4e4;
+// a team's CTAs have at least this many rows of kTeamRow carriers each (the
+// step of an 829-carrier event no longer shortens beyond 52 CTAs)
+constexpr int kTeamMinRows = 4;
 constexpr int kMaxUnits = 1 << 16;
 constexpr int kMaxSymUnits = 1 << 18;  // units of one step of the symmetric kernel
 // upload_sym_plan: the plan needs more units or tiles than the buffers hold
@@ -179,6 +197,11 @@ struct sim_t {
   int32_t* d_sym_ctr = nullptr;     // partials written per tile
   SymStep* d_sym_rec = nullptr;
   int32_t* d_sym_ready = nullptr;
+
+  TeamEntry* d_team = nullptr;  // the team kernel's CTAs [sm_count]
+  TeamEntry* h_team = nullptr;
+  int team_grid = 0;        // CTAs of the current chunk (0: another kernel runs)
+  size_t team_smem = 0;     // their dynamic shared memory
 
   // host state
   std::vector<HostSlot> slots;
@@ -759,14 +782,69 @@ int upload_units(sim_t* s, bool allow_split, bool slot_major = false) {
   return SIM_OK;
 }
 
+// Plan the team kernel for the running slots and upload it: every event a
+// team of CTAs in proportion to its pair work.  *fits is false when there are
+// more events than SMs or an event's positions exceed a CTA's shared memory.
+int plan_team(sim_t* s, bool* fits) {
+  *fits = false;
+  struct Ev {
+    int slot, size, most;
+    double work;
+  };
+  std::vector<Ev> ev;
+  const int P = s->sm_count;
+  for (int k = 0; k < s->S; ++k) {
+    const HostSlot& h = s->slots[k];
+    if (!h.used || !h.running) continue;
+    const int n = h.n_h + h.n_e;
+    Ev e{k, 1, 1, (double)n * (double)n};
+    while (e.size <= P && team_smem_bytes(h.n_h, h.n_e, e.size) > kTeamSmem) ++e.size;
+    if (e.size > P) return SIM_OK;
+    const int rows = (h.n_h + kTeamRow - 1) / kTeamRow + (h.n_e + kTeamRow - 1) / kTeamRow;
+    e.most = std::max(e.size, rows / kTeamMinRows);
+    ev.push_back(e);
+  }
+  TeamEntry* out = s->h_team;
+  int64_t need = 0;
+  for (const Ev& e : ev) need += e.size;
+  if (ev.empty() || need > P) return SIM_OK;
+  // one CTA more at a time for the event whose CTAs have the most work
+  auto load = [](const Ev& e) { return e.size < e.most ? e.work / e.size : 0.0; };
+  std::vector<std::pair<double, int>> heap;
+  for (size_t q = 0; q < ev.size(); ++q) heap.push_back({load(ev[q]), (int)q});
+  std::make_heap(heap.begin(), heap.end());
+  for (int left = P - (int)need; left > 0 && heap.front().first > 0.0; --left) {
+    std::pop_heap(heap.begin(), heap.end());
+    Ev& e = ev[heap.back().second];
+    ++e.size;
+    heap.back().first = load(e);
+    std::push_heap(heap.begin(), heap.end());
+  }
+  int grid = 0;
+  for (const Ev& e : ev)
+    for (int q = 0; q < e.size; ++q) out[grid++] = TeamEntry{e.slot, q, e.size, 0};
+  int64_t smem = 0;
+  for (const Ev& e : ev) {
+    const HostSlot& h = s->slots[e.slot];
+    smem = std::max(smem, team_smem_bytes(h.n_h, h.n_e, e.size));
+  }
+  s->team_grid = grid;
+  s->team_smem = (size_t)smem;
+  CK(h2d(s, s->d_team, s->h_team, grid * sizeof(TeamEntry)));
+  *fits = true;
+  return SIM_OK;
+}
+
 // Issue one chunk: K fused steps (one launch per chunk, or one per step), or
 // in PLAIN mode field + update launches for one step; then the close kernel
 // and the summary copy.
 int issue_chunk(sim_t* s, int K, bool multi) {
   const bool plain = s->opt.mode == CTS_MODE_PLAIN;
-  CK(cudaMemsetAsync(s->d_unit_counter, 0, K * sizeof(int32_t), s->stream));
   CK(cudaMemsetAsync(s->d_ret, 0, (size_t)K * s->S * 2 * sizeof(int32_t), s->stream));
-  CK(cudaMemsetAsync(s->d_tiles_done, 0, (size_t)K * s->S * sizeof(int32_t), s->stream));
+  if (s->team_grid == 0) {
+    CK(cudaMemsetAsync(s->d_unit_counter, 0, K * sizeof(int32_t), s->stream));
+    CK(cudaMemsetAsync(s->d_tiles_done, 0, (size_t)K * s->S * sizeof(int32_t), s->stream));
+  }
   if (s->sym)
     CK(cudaMemsetAsync(s->d_sym_ready, 0, (size_t)K * s->S * sizeof(int32_t), s->stream));
   if (s->d_induced)
@@ -800,7 +878,11 @@ int issue_chunk(sim_t* s, int K, bool multi) {
     // inside a stream capture the events become external event-record nodes
     const unsigned evflag = capturing(s) ? cudaEventRecordExternal : cudaEventRecordDefault;
     if (timed) CK(cudaEventRecordWithFlags(s->lev[0], s->stream, evflag));
-    if (multi) {
+    if (s->team_grid > 0) {
+      CK(launch_team(a, s->d_team, 0, K, s->team_grid, s->team_smem, s->stream));
+      if (timed) CK(cudaEventRecordWithFlags(s->lev[1], s->stream, evflag));
+      s->st_launch += 1;
+    } else if (multi) {
       CK(launch_step(s->variant, a, 0, K, s->grid, s->stream));
       if (timed) CK(cudaEventRecordWithFlags(s->lev[1], s->stream, evflag));
       s->st_launch += 1;
@@ -829,6 +911,8 @@ int run_chunk(sim_t* s) {
   NvtxRange range("cts chunk");
   const bool plain = s->opt.mode == CTS_MODE_PLAIN;
   const int K = plain ? 1 : s->K;
+  bool team = false;
+  s->team_grid = 0;
   if (plain) {
     // the update launch walks the running slot listed in d_list
     int n = 0;
@@ -850,17 +934,24 @@ int run_chunk(sim_t* s) {
     // pair work fills the GPU, the per-pair kernel (finer work units, shorter
     // steps) below it; the events' state is the same for both
     double W = 0.0;
-    int max_tiles = 0;
+    int max_tiles = 0, max_n = 0;
     for (auto& h : s->slots)
       if (h.used && h.running) {
         W += (double)(h.n_h + h.n_e) * (double)(h.n_h + h.n_e);
+        max_n = std::max(max_n, h.n_h + h.n_e);
         max_tiles = std::max(max_tiles, (h.n_h + kSymTile - 1) / kSymTile +
                                             (h.n_e + kSymTile - 1) / kSymTile);
       }
     const bool serve = s->opt.mode == CTS_MODE_SERVE;
     const int sym_v = (serve || max_tiles > kSymLargeTiles) ? kSymVariantLarge : kSymVariant;
-    int rcv = set_variant(s, W >= (serve ? kSymMinWorkServe : kSymMinWork) ? sym_v : kPairVariant);
+    const bool full = W >= (serve ? kSymMinWorkServe : kSymMinWork);
+    int rcv = set_variant(s, full ? sym_v : kPairVariant);
     if (rcv) return rcv;
+    if (!serve && W < kTeamMaxLoad * max_n && !full && !s->field.spherical &&
+        !s->opt.step_launches) {
+      rcv = plan_team(s, &team);
+      if (rcv) return rcv;
+    }
   }
   // one launch for the whole chunk: the queue replays the step's pieces K
   // times, slot by slot
@@ -879,12 +970,14 @@ int run_chunk(sim_t* s) {
   const bool multi = !plain && !sph && s->dynamic && (s->sym || s->ph.repulsion) &&
                      !s->opt.step_launches;
   // PLAIN splits tiles too: one event alone must still spread over the SMs
-  if (!sph && !s->sym) rc = upload_units(s, true, multi);
+  if (!sph && !s->sym && !team) rc = upload_units(s, true, multi);
   if (rc) return rc;
   const int gi = sph ? 2 * variant_count() : 2 * s->variant + (multi ? 1 : 0);
-  const int nl = (multi || sph) ? 1 : K;  // step-kernel launches in the chunk
+  const int nl = (multi || sph || team) ? 1 : K;  // step-kernel launches in the chunk
   CK(cudaEventRecord(s->ev0, s->stream));
-  if (!plain && !s->opt.disable_graphs) {
+  // (the team kernel's grid and shared memory follow the running events: it is
+  // launched directly)
+  if (!plain && !team && !s->opt.disable_graphs) {
     cudaGraphExec_t& graph = s->graphs[gi];
     if (!graph || s->graph_K[gi] != K) {
       if (graph) {
@@ -919,7 +1012,7 @@ int run_chunk(sim_t* s) {
   s->st_ms += ms;
   if (s->opt.time_launches && !plain) {
     double pairs = 0.0;
-    if (s->sym) {
+    if (s->sym || team) {
       for (const HostSlot& h : s->slots)
         if (h.used && h.running && h.n_h > 0) pairs += (double)(h.n_h + h.n_e) * (h.n_h + h.n_e);
     } else {
@@ -1243,6 +1336,8 @@ int alloc_all(sim_t* s) {
   AL(s->d_sym_ctr, s->sym_tiles_cap);
   AL(s->d_sym_rec, (int64_t)kMaxK * s->S);
   AL(s->d_sym_ready, (int64_t)kMaxK * s->S);
+  AL(s->d_team, s->sm_count);
+  HL(s->h_team, s->sm_count);
 
   HL(s->h_sym_units, kMaxSymUnits);
   HL(s->h_sym_nu, 1);
@@ -1282,12 +1377,12 @@ void free_all(sim_t* s) {
                  s->d_combine, s->d_tiles_done, s->d_induced, s->d_err, s->d_field, s->d_explicit,
                  s->d_list, s->d_drift, s->d_induced_px, s->d_sym_units, s->d_sym_nu,
                  s->d_sym_tiles, s->d_sym_lists, s->d_sym_part, s->d_sym_ctr, s->d_sym_rec,
-                 s->d_sym_ready};
+                 s->d_sym_ready, s->d_team};
   for (void* p : dev)
     if (p) cudaFree(p);
   void* host[] = {s->h_summary, s->h_units, s->h_cta_begin, s->h_list, s->h_slotdev, s->h_readout,
                   s->h_pixels, s->h_err, s->h_induced, s->h_induced_px, s->h_sym_units,
-                  s->h_sym_nu, s->h_sym_tiles, s->h_sym_lists};
+                  s->h_sym_nu, s->h_sym_tiles, s->h_sym_lists, s->h_team};
   for (void* p : host)
     if (p) cudaFreeHost(p);
   if (s->ev0) cudaEventDestroy(s->ev0);
@@ -1422,6 +1517,7 @@ int sim_init(const sim_sensor_t* sensor, const sim_field_t* field, const sim_mob
     }
   }
   if (!rc) rc = set_variant(s, choose_variant(s));
+  if (!rc && team_prepare() != cudaSuccess) rc = SIM_ECUDA;
   if (!rc && s->field.spherical) {
     if (spherical_prepare() != cudaSuccess) rc = SIM_ECUDA;
     else s->sph_cluster = spherical_cluster(s->S, s->opt.sph_cluster);
