@@ -304,13 +304,16 @@ cudaError_t launch_team(const StepArgs& a, const TeamEntry* ctas, int k0, int nk
                         size_t smem, cudaStream_t s);
 cudaError_t launch_update(const StepArgs& a, int k, int n_slots_list, const int32_t* slot_list,
                           int grid, cudaStream_t s);
+// most: carriers of the largest listed slot.  launch_init also clears the
+// slots' pixel maps and readout counts, launch_bin adds to them.
 cudaError_t launch_init(const Phys& ph, Arena A, SlotDev* slots, const int32_t* slot_list,
-                        int n, const ExplicitRec* explicit_buf, cudaStream_t s);
+                        int n, int most, const ExplicitRec* explicit_buf, int32_t* pixels,
+                        SlotReadout* readout, cudaStream_t s);
 cudaError_t launch_close(const Phys& ph, Arena A, SlotDev* slots, const int32_t* slot_list,
                          int n, const int32_t* ret, int S, int K, SlotSummary* summary,
                          cudaStream_t s);
 cudaError_t launch_bin(const Phys& ph, Arena A, const SlotDev* slots, const int32_t* slot_list,
-                       int n, int32_t* pixels, SlotReadout* readout, cudaStream_t s);
+                       int n, int most, int32_t* pixels, SlotReadout* readout, cudaStream_t s);
 cudaError_t launch_bin_points(const Phys& ph, const double* x, const double* y, int64_t n,
                               int32_t* pixels, long long* outside, cudaStream_t s);
 // Simplified spherical model: one cluster of `cluster` CTAs (1, 2 or 4) per

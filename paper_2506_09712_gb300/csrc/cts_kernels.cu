@@ -323,7 +323,19 @@ __device__ __forceinline__ int pixel_at(double pitch, int grid_n, double x, doub
   return (int)fy * grid_n + (int)fx;
 }
 
+// The same for the binning kernels: FP32 decides a carrier that lies further
+// from every pixel edge than its rounding (1e-5 of a pixel and of |x| / pitch,
+// against 2^-23 of them), the FP64 divisions (slow on this GPU) the others.
 __device__ __forceinline__ int pixel_key(const Phys& ph, double x, double y) {
+  const float inv = 1.0f / (float)ph.pitch, half = 0.5f * (float)ph.grid_n;
+  const float n = (float)ph.grid_n;
+  const float tx = fmaf((float)x, inv, half), ty = fmaf((float)y, inv, half);
+  const float gx = 1e-5f * (1.0f + half + fabsf(tx)), gy = 1e-5f * (1.0f + half + fabsf(ty));
+  const float fx = floorf(tx), fy = floorf(ty);
+  if (tx - fx > gx && fx + 1.0f - tx > gx && ty - fy > gy && fy + 1.0f - ty > gy) {  // not NaN
+    if (!(fx >= 0.0f && fy >= 0.0f && fx < n && fy < n)) return -1;
+    return (int)fy * ph.grid_n + (int)fx;
+  }
   return pixel_at(ph.pitch, ph.grid_n, x, y);
 }
 
@@ -2046,6 +2058,7 @@ __global__ void update_kernel(StepArgs a, int k, const int32_t* slot_list, int n
 // Block-wide order-preserving compaction of one species range (in place).
 // ---------------------------------------------------------------------------
 constexpr int kAuxThreads = 256;
+constexpr int kCloseThreads = 1024;
 
 __device__ int block_exclusive_scan(int v, int* warp_sums, int* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -2053,14 +2066,16 @@ __device__ int block_exclusive_scan(int v, int* warp_sums, int* total) {
   const int within = __popc(m & ((1u << lane) - 1u));
   if (lane == 0) warp_sums[warp] = __popc(m);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int acc = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      const int t = warp_sums[w];
-      warp_sums[w] = acc;
-      acc += t;
+  if (warp == 0) {
+    const int mine = lane < (int)(blockDim.x >> 5) ? warp_sums[lane] : 0;
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
     }
-    *total = acc;
+    warp_sums[lane] = incl - mine;
+    if (lane == 31) *total = incl;
   }
   __syncthreads();
   return warp_sums[warp] + within;
@@ -2101,11 +2116,15 @@ __device__ int compact_range(const Arena& A, int64_t start, int n, int64_t rbase
   return out;
 }
 
-__global__ void __launch_bounds__(kAuxThreads) close_kernel(Phys ph, Arena A, SlotDev* slots,
-                                                            const int32_t* ret, int S_count, int K,
-                                                            SlotSummary* summary) {
-  __shared__ int warp_sums[kAuxThreads / 32];
+// One CTA per slot.  Bound: latency (a finished or idle slot: one load; a
+// running one: its retire counts, then one pass of loads, a scan and stores
+// per 1024 carriers).
+__global__ void __launch_bounds__(kCloseThreads) close_kernel(Phys ph, Arena A, SlotDev* slots,
+                                                              const int32_t* ret, int S_count,
+                                                              int K, SlotSummary* summary) {
+  __shared__ int warp_sums[32];
   __shared__ int total;
+  __shared__ int s_ret[2];
   const int slot = blockIdx.x;
   SlotDev* S = slots + slot;
   SlotSummary sm{};
@@ -2128,11 +2147,16 @@ __global__ void __launch_bounds__(kAuxThreads) close_kernel(Phys ph, Arena A, Sl
     return;
   }
 #endif
-  int nah = S->act_h, nae = S->act_e;
-  for (int kk = 0; kk < K; ++kk) {
-    nah -= ret[((int64_t)kk * S_count + slot) * 2 + 0];
-    nae -= ret[((int64_t)kk * S_count + slot) * 2 + 1];
+  if (threadIdx.x < 64) {  // warp w: species w's retired carriers of the chunk
+    const int w = threadIdx.x >> 5;
+    int sum = 0;
+    for (int kk = threadIdx.x & 31; kk < K; kk += 32)
+      sum += ret[((int64_t)kk * S_count + slot) * 2 + w];
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if ((threadIdx.x & 31) == 0) s_ret[w] = sum;
   }
+  __syncthreads();
+  const int nah = S->act_h - s_ret[0], nae = S->act_e - s_ret[1];
   int done = 0, status = 0;
   if (S->flags & kErrNumeric) {
     done = 1;
@@ -2178,72 +2202,52 @@ __global__ void __launch_bounds__(kAuxThreads) close_kernel(Phys ph, Arena A, Sl
 }
 
 // ---------------------------------------------------------------------------
-// Initial cloud (Algorithm 1, first step; Eq. 2), one CTA per new slot.
+// Initial cloud (Algorithm 1, first step; Eq. 2).  Bound: FP64 arithmetic (the
+// Box-Muller normals; two FP64 lanes per clock and SM), so the carriers of a
+// slot are spread over CTAs of kInitThreads (blockIdx.x; blockIdx.y is the
+// slot's place in the list) and a pair's hole and electron, which start at the
+// same point, share one draw.  The host has put the slot's counts as if every
+// carrier stayed (place_event); the few that do not are taken off here.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kAuxThreads) init_kernel(Phys ph, Arena A, SlotDev* slots,
-                                                           const int32_t* slot_list,
-                                                           const ExplicitRec* ex) {
-  __shared__ int ret_h, ret_e;
-  SlotDev* S = slots + slot_list[blockIdx.x];
-  if (threadIdx.x == 0) {
-    ret_h = 0;
-    ret_e = 0;
-  }
-  __syncthreads();
-  const int np = S->n_pairs;
+constexpr int kInitThreads = 64;
+
+__global__ void __launch_bounds__(kInitThreads) init_kernel(Phys ph, Arena A, SlotDev* slots,
+                                                            const int32_t* slot_list,
+                                                            const ExplicitRec* ex, int32_t* pixels,
+                                                            SlotReadout* readout) {
+  const int slot = slot_list[blockIdx.y];
+  SlotDev* S = slots + slot;
+  const int np = S->n_pairs, kind = S->kind, cap_h = S->cap_h, cap_e = S->cap_e;
   const double H = ph.H;
   const double sigma = S->sigma_um >= 0.0 ? S->sigma_um : 0.0044 * pow(S->energy_keV, 1.75);
   const double z_entry = H - S->depth_um;
-  const double th = S->theta_deg * (M_PI / 180.0), phi = S->phi_deg * (M_PI / 180.0);
-  const double ux = sin(th) * cos(phi), uy = sin(th) * sin(phi), uz = -cos(th);
-  const double axv = cos(th) * cos(phi), ayv = cos(th) * sin(phi), azv = sin(th);
-  const double bxv = -sin(phi), byv = cos(phi);
+  double ux = 0.0, uy = 0.0, uz = 0.0, axv = 0.0, ayv = 0.0, azv = 0.0, bxv = 0.0, byv = 0.0;
+  if (kind == 1) {
+    const double th = S->theta_deg * (M_PI / 180.0), phi = S->phi_deg * (M_PI / 180.0);
+    ux = sin(th) * cos(phi), uy = sin(th) * sin(phi), uz = -cos(th);
+    axv = cos(th) * cos(phi), ayv = cos(th) * sin(phi), azv = sin(th);
+    bxv = -sin(phi), byv = cos(phi);
+  }
   // frame anchor: the absorption point, or the midpoint of a track
-  const double half = S->kind == 1 ? 0.5 * S->track_len_um : 0.0;
+  const double half = kind == 1 ? 0.5 * S->track_len_um : 0.0;
   const double ax0 = S->x0 + half * ux, ay0 = S->y0 + half * uy;
-  const double az0 = fmin(fmax(S->kind == 1 ? H + half * uz : z_entry, 0.0), H);
-  const int total_entries = S->cap_h + S->cap_e;
+  const double az0 = fmin(fmax(kind == 1 ? H + half * uz : z_entry, 0.0), H);
+  const int total_entries = cap_h + cap_e;
 #ifdef CTS_BOUNDS_CHECK
   // the slot's range, the explicit records it reads, and every carrier id
-  __shared__ int bad;
-  if (threadIdx.x == 0)
-    bad = !slot_in_arena(A, S) || S->n_pairs < 0 || S->n_pairs > S->cap_h ||
-          (S->kind == 2 && (S->explicit_off < 0 || S->explicit_off + total_entries > A.capacity));
-  __syncthreads();
-  const int loop_end = bad ? 0 : total_entries;
-#else
-  const int loop_end = total_entries;
+  if (!slot_in_arena(A, S) || np < 0 || np > cap_h + (kind == 2 ? cap_e : 0) ||
+      (kind != 2 && cap_e != 0 && cap_e != np) ||
+      (kind == 2 && (S->explicit_off < 0 || S->explicit_off + total_entries > A.capacity))) {
+    if (threadIdx.x == 0) atomicOr(&S->flags, kErrBounds);
+    return;
+  }
 #endif
-
-  for (int e = threadIdx.x; e < loop_end; e += blockDim.x) {
-    const int spec = e < S->cap_h ? 0 : 1;
-    const int64_t idx = S->base + e;
-    double x, y, z;
-    int id;
-    if (S->kind == 2) {
-      const ExplicitRec r = ex[S->explicit_off + e];
-      x = r.x; y = r.y; z = r.z; id = r.cid;
-    } else {
-      const int pidx = spec ? e - S->cap_h : e;
-      id = spec ? np + pidx : pidx;
-      const double3 n = normals_d(stream_words(S->seed, S->event_id, 1u, (uint32_t)pidx, 0u));
-      if (S->kind == 1) {
-        const uint4 w = stream_words(S->seed, S->event_id, 1u, (uint32_t)pidx, 1u);
-        const double s = uniform_d(w.x) * S->track_len_um;
-        x = S->x0 + s * ux + sigma * (n.x * axv + n.y * bxv);
-        y = S->y0 + s * uy + sigma * (n.x * ayv + n.y * byv);
-        z = H + s * uz + sigma * (n.x * azv);
-      } else {
-        x = S->x0 + sigma * n.x;
-        y = S->y0 + sigma * n.y;
-        z = z_entry + sigma * n.z;
-      }
-    }
-    const int64_t rid = S->base + id;
+  auto put = [&](int spec, int e, int id, double x, double y, double z) {
+    const int64_t idx = S->base + e, rid = S->base + id;
 #ifdef CTS_BOUNDS_CHECK
     if (id < 0 || id >= total_entries) {
       atomicOr(&S->flags, kErrBounds);
-      continue;
+      return;
     }
 #endif
     int state = kStateActive;
@@ -2263,33 +2267,47 @@ __global__ void __launch_bounds__(kAuxThreads) init_kernel(Phys ph, Arena A, Slo
     A.fx[rid] = state == kStateCollected ? x : __longlong_as_double(0x7ff8000000000000LL);
     A.fy[rid] = state == kStateCollected ? y : __longlong_as_double(0x7ff8000000000000LL);
     if (state != kStateActive) {
-      atomicAdd(spec ? &ret_e : &ret_h, 1);
+      atomicSub(spec ? &S->act_e : &S->act_h, 1);
       A.sh[0][idx] = make_float4(kParked, kParked, kParked, 0.0f);
     } else {
       A.sh[0][idx] = make_float4((float)(x - ax0), (float)(y - ay0), (float)(z - az0), 0.0f);
     }
     A.sh[1][idx] = make_float4(kParked, kParked, kParked, 0.0f);  // no step's entry yet
+  };
+  // explicit records one by one; generated pairs: the hole and its electron
+  const int n = kind == 2 ? total_entries : np;
+  for (int e = blockIdx.x * kInitThreads + threadIdx.x; e < n; e += gridDim.x * kInitThreads) {
+    if (kind == 2) {
+      const ExplicitRec r = ex[S->explicit_off + e];
+      put(e < cap_h ? 0 : 1, e, r.cid, r.x, r.y, r.z);
+      continue;
+    }
+    const double3 g = normals_d(stream_words(S->seed, S->event_id, 1u, (uint32_t)e, 0u));
+    double x, y, z;
+    if (kind == 1) {
+      const uint4 w = stream_words(S->seed, S->event_id, 1u, (uint32_t)e, 1u);
+      const double s = uniform_d(w.x) * S->track_len_um;
+      x = S->x0 + s * ux + sigma * (g.x * axv + g.y * bxv);
+      y = S->y0 + s * uy + sigma * (g.x * ayv + g.y * byv);
+      z = H + s * uz + sigma * (g.x * azv);
+    } else {
+      x = S->x0 + sigma * g.x;
+      y = S->y0 + sigma * g.y;
+      z = z_entry + sigma * g.z;
+    }
+    put(0, e, e, x, y, z);
+    if (cap_e > 0) put(1, cap_h + e, np + e, x, y, z);
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  // the slot's record and its (empty) readout
+  const int npix = ph.grid_n * ph.grid_n;
+  for (int p = blockIdx.x * kInitThreads + threadIdx.x; p < npix; p += gridDim.x * kInitThreads)
+    pixels[(int64_t)slot * npix + p] = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    readout[slot] = SlotReadout{};
     S->ax = ax0;
     S->ay = ay0;
     S->az[0][0] = S->az[0][1] = az0;
     S->az[1][0] = S->az[1][1] = az0;
-    S->n_h = S->cap_h;
-    S->n_e = S->cap_e;
-    S->act_h = S->cap_h - ret_h;
-    S->act_e = S->cap_e - ret_e;
-    S->step0 = 0;
-    S->n_steps = 0;
-#ifdef CTS_BOUNDS_CHECK
-    S->flags = (bad || (S->flags & kErrBounds)) ? kErrBounds : 0;
-#else
-    S->flags = 0;
-#endif
-    S->status = 0;
-    S->interactions = 0ull;
-    S->running = 1;
   }
 }
 
@@ -2308,15 +2326,16 @@ __device__ __forceinline__ void warp_count(int key, int32_t* pix, int* outside) 
   }
 }
 
+// blockIdx.y: the slot's place in the list; its carriers spread over
+// blockIdx.x.  Adds to the slot's counts, which init_kernel cleared.
 __global__ void __launch_bounds__(kAuxThreads) bin_kernel(Phys ph, Arena A, const SlotDev* slots,
                                                           const int32_t* slot_list,
                                                           int32_t* pixels, SlotReadout* readout) {
   __shared__ int outside, collected, lost;
-  const int slot = slot_list[blockIdx.x];
+  const int slot = slot_list[blockIdx.y];
   const SlotDev* S = slots + slot;
   const int npix = ph.grid_n * ph.grid_n;
   int32_t* pix = pixels + (int64_t)slot * npix;
-  for (int t = threadIdx.x; t < npix; t += blockDim.x) pix[t] = 0;
   if (threadIdx.x == 0) outside = collected = lost = 0;
   __syncthreads();
 #ifdef CTS_BOUNDS_CHECK
@@ -2324,27 +2343,32 @@ __global__ void __launch_bounds__(kAuxThreads) bin_kernel(Phys ph, Arena A, cons
 #else
   const int n = S->n_total;
 #endif
-  const int n_round = (n + blockDim.x - 1) / blockDim.x * blockDim.x;
-  for (int id = threadIdx.x; id < n_round; id += blockDim.x) {
+  const int stride = gridDim.x * blockDim.x;
+  for (int i0 = blockIdx.x * blockDim.x; i0 < n; i0 += stride) {
+    const int id = i0 + threadIdx.x;
     int key = -2;
+    bool gone = false, moving = false;
     if (id < n) {
       const int8_t st = A.cstate[S->base + id];
-      if ((st & kStateMask) == kStateCollected) {
-        key = pixel_key(ph, A.fx[S->base + id], A.fy[S->base + id]);
-        atomicAdd(&collected, 1);
-      } else if ((st & kStateMask) == kStateActive && (st & kElectronBit)) {
-        atomicAdd(&lost, 1);
-      }
+      gone = (st & kStateMask) == kStateCollected;
+      moving = (st & kStateMask) == kStateActive && (st & kElectronBit);
+      if (gone) key = pixel_key(ph, A.fx[S->base + id], A.fy[S->base + id]);
     }
     warp_count(key, pix, &outside);
+    const unsigned mg = __ballot_sync(0xffffffffu, gone), mm = __ballot_sync(0xffffffffu, moving);
+    if ((threadIdx.x & 31) == 0) {
+      if (mg) atomicAdd(&collected, __popc(mg));
+      if (mm) atomicAdd(&lost, __popc(mm));
+    }
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    SlotReadout r{};
-    r.n_collected = collected;
-    r.n_outside = outside;
-    r.n_lost = lost;
-    readout[slot] = r;
+    auto add = [](long long* p, int v) {
+      if (v) atomicAdd(reinterpret_cast<unsigned long long*>(p), (unsigned long long)v);
+    };
+    add(&readout[slot].n_collected, collected);
+    add(&readout[slot].n_outside, outside);
+    add(&readout[slot].n_lost, lost);
   }
 }
 
@@ -3090,9 +3114,13 @@ cudaError_t launch_update(const StepArgs& a, int k, int n_slots_list, const int3
 }
 
 cudaError_t launch_init(const Phys& ph, Arena A, SlotDev* slots, const int32_t* slot_list, int n,
-                        const ExplicitRec* explicit_buf, cudaStream_t s) {
+                        int most, const ExplicitRec* explicit_buf, int32_t* pixels,
+                        SlotReadout* readout, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  init_kernel<<<n, kAuxThreads, 0, s>>>(ph, A, slots, slot_list, explicit_buf);
+  // one carrier pair per thread, at most 4096 CTAs per event
+  const int per = most < kInitThreads ? 1 : (most + kInitThreads - 1) / kInitThreads;
+  init_kernel<<<dim3(per < 4096 ? per : 4096, n), kInitThreads, 0, s>>>(
+      ph, A, slots, slot_list, explicit_buf, pixels, readout);
   return cudaGetLastError();
 }
 
@@ -3100,14 +3128,16 @@ cudaError_t launch_close(const Phys& ph, Arena A, SlotDev* slots, const int32_t*
                          int n, const int32_t* ret, int S, int K, SlotSummary* summary,
                          cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  close_kernel<<<n, kAuxThreads, 0, s>>>(ph, A, slots, ret, S, K, summary);
+  close_kernel<<<n, kCloseThreads, 0, s>>>(ph, A, slots, ret, S, K, summary);
   return cudaGetLastError();
 }
 
 cudaError_t launch_bin(const Phys& ph, Arena A, const SlotDev* slots, const int32_t* slot_list,
-                       int n, int32_t* pixels, SlotReadout* readout, cudaStream_t s) {
+                       int n, int most, int32_t* pixels, SlotReadout* readout, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  bin_kernel<<<n, kAuxThreads, 0, s>>>(ph, A, slots, slot_list, pixels, readout);
+  const int per = most < kAuxThreads ? 1 : (most + kAuxThreads - 1) / kAuxThreads;
+  bin_kernel<<<dim3(per < 1024 ? per : 1024, n), kAuxThreads, 0, s>>>(ph, A, slots, slot_list,
+                                                                      pixels, readout);
   return cudaGetLastError();
 }
 

@@ -453,6 +453,11 @@ int place_event(sim_t* s, int slot, EventRec&& r, int64_t base) {
   d.cap_h = r.cap_h;
   d.cap_e = r.cap_e;
   d.n_total = r.cap_h + r.cap_e;
+  // every carrier present and active: init_kernel takes off the ones that
+  // start beyond a surface
+  d.n_h = d.act_h = r.cap_h;
+  d.n_e = d.act_e = r.cap_e;
+  d.running = 1;
   d.kind = r.ev.kind;
   d.n_pairs = r.n_pairs;
   d.energy_keV = r.ev.energy_keV;
@@ -523,15 +528,17 @@ int admit(sim_t* s) {
 }
 
 int launch_inits(sim_t* s) {
-  int n = 0;
+  int n = 0, most = 0;
   for (int k = 0; k < s->S; ++k)
     if (s->slots[k].used && s->slots[k].needs_init) {
       s->h_list[n++] = k;
       s->slots[k].needs_init = false;
+      most = std::max(most, s->slots[k].rec.cap_h + s->slots[k].rec.cap_e);
     }
   if (!n) return SIM_OK;
   CK(h2d(s, s->d_list, s->h_list, n * sizeof(int32_t)));
-  CK(launch_init(s->ph, s->A, s->d_slots, s->d_list, n, s->d_explicit, s->stream));
+  CK(launch_init(s->ph, s->A, s->d_slots, s->d_list, n, most, s->d_explicit, s->d_pixels,
+                 s->d_readout, s->stream));
   // keep h_list stable until the copy has been consumed
   CK(cudaStreamSynchronize(s->stream));
   s->st_launch += 1;
@@ -1188,10 +1195,14 @@ int pump(sim_t* s, bool defer, bool* progressed) {
     }
   }
   if (fin.empty()) return SIM_OK;
-  for (size_t q = 0; q < fin.size(); ++q) s->h_list[q] = fin[q];
+  int most = 0;
+  for (size_t q = 0; q < fin.size(); ++q) {
+    s->h_list[q] = fin[q];
+    most = std::max(most, s->slots[fin[q]].rec.cap_h + s->slots[fin[q]].rec.cap_e);
+  }
   CK(h2d(s, s->d_list, s->h_list, fin.size() * sizeof(int32_t)));
-  CK(launch_bin(s->ph, s->A, s->d_slots, s->d_list, (int)fin.size(), s->d_pixels, s->d_readout,
-                s->stream));
+  CK(launch_bin(s->ph, s->A, s->d_slots, s->d_list, (int)fin.size(), most, s->d_pixels,
+                s->d_readout, s->stream));
   s->st_launch += 1;
   if (defer) {
     CK(cudaStreamSynchronize(s->stream));
