@@ -147,8 +147,9 @@ typedef struct sim_options_t {
                               sim_init when it matches this device and build,
                               written by sim_autotune; NULL = none */
   int32_t sph_cluster;     /* spherical model: CTAs per event (1, 2 or 4); 0 =
-                              the widest with which all max_slots events are
-                              resident at once.  Results do not depend on it. */
+                              the widest with which the running events are
+                              resident at once, chosen per chunk.  Results do
+                              not depend on it. */
   int32_t reserved;
 } sim_options_t;
 

@@ -2446,7 +2446,8 @@ __device__ __forceinline__ int sph_shift(unsigned long long lo, unsigned long lo
 }
 
 template <bool PX>
-__global__ void __launch_bounds__(1024, 1) spherical_kernel(StepArgs a, int k0, int nk) {
+__global__ void __launch_bounds__(1024, 1) spherical_kernel(StepArgs a, const int32_t* slot_list,
+                                                            int k0, int nk) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
@@ -2465,8 +2466,7 @@ __global__ void __launch_bounds__(1024, 1) spherical_kernel(StepArgs a, int k0, 
   __shared__ unsigned long long s_rng[2];  // the keys' range: this step's, being found
   __shared__ unsigned long long s_lo;      // the bins' range
   __shared__ int s_shift;
-  const int slot = blockIdx.x / C;
-  if (slot >= a.S) return;
+  const int slot = slot_list[blockIdx.x / C];
   SlotDev* S = a.slots + slot;
   if (!S->running) return;
   const int nh = S->n_h;
@@ -3193,22 +3193,23 @@ int spherical_cluster(int slots, int request) {
   return 1;
 }
 
-cudaError_t launch_spherical(const StepArgs& a, int k0, int nk, int cluster, cudaStream_t s) {
-  if (a.S <= 0) return cudaSuccess;
+cudaError_t launch_spherical(const StepArgs& a, const int32_t* slot_list, int n, int k0, int nk,
+                             int cluster, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)cluster;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3((unsigned)(a.S * cluster), 1, 1);
+  cfg.gridDim = dim3((unsigned)(n * cluster), 1, 1);
   cfg.blockDim = dim3(1024, 1, 1);
   cfg.dynamicSmemBytes = kSphSmem;
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (a.induced_px) return cudaLaunchKernelEx(&cfg, spherical_kernel<true>, a, k0, nk);
-  return cudaLaunchKernelEx(&cfg, spherical_kernel<false>, a, k0, nk);
+  if (a.induced_px) return cudaLaunchKernelEx(&cfg, spherical_kernel<true>, a, slot_list, k0, nk);
+  return cudaLaunchKernelEx(&cfg, spherical_kernel<false>, a, slot_list, k0, nk);
 }
 
 cudaError_t launch_generate(const GenEvent* ev, int n_events, double pitch_um, int grid_n,

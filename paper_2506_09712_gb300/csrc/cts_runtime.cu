@@ -234,6 +234,7 @@ struct sim_t {
   std::vector<int> table_var;
   int base_variant = 0;
   int sph_cluster = 1;  // CTAs per event of the spherical model
+  int sph_n = 0;        // running events of the current chunk (listed in d_list)
   std::string autotune_cache;  // copied from the options
   std::string device_name;
 
@@ -865,7 +866,7 @@ int issue_chunk(sim_t* s, int K, bool multi) {
     const bool timed = s->opt.time_launches != 0 && !plain;
     const unsigned evflag = capturing(s) ? cudaEventRecordExternal : cudaEventRecordDefault;
     if (timed) CK(cudaEventRecordWithFlags(s->lev[0], s->stream, evflag));
-    CK(launch_spherical(a, 0, K, s->sph_cluster, s->stream));
+    CK(launch_spherical(a, s->d_list, s->sph_n, 0, K, s->sph_cluster, s->stream));
     if (timed) CK(cudaEventRecordWithFlags(s->lev[1], s->stream, evflag));
     s->st_launch += 1;
   } else if (plain) {
@@ -920,12 +921,19 @@ int run_chunk(sim_t* s) {
   const int K = plain ? 1 : s->K;
   bool team = false;
   s->team_grid = 0;
-  if (plain) {
-    // the update launch walks the running slot listed in d_list
+  const bool sph = s->field.spherical != 0;
+  if (plain || sph) {
+    // the update launch walks the running slot listed in d_list, the
+    // spherical kernel's clusters take one listed slot each
     int n = 0;
     for (int k = 0; k < s->S; ++k)
       if (s->slots[k].used && s->slots[k].running) s->h_list[n++] = k;
     CK(h2d(s, s->d_list, s->h_list, std::max(n, 1) * sizeof(int32_t)));
+    s->sph_n = n;
+    // the widest cluster with which the events of this chunk are resident at
+    // once (the results do not depend on it): on 64 20 keV events 40 us per
+    // step with 2 CTAs per event against 62 us with 1
+    if (sph && s->opt.sph_cluster == 0) s->sph_cluster = spherical_cluster(n, 0);
   }
   if (!plain && !s->table_min.empty()) {
     double W = 0.0;
@@ -962,7 +970,6 @@ int run_chunk(sim_t* s) {
   }
   // one launch for the whole chunk: the queue replays the step's pieces K
   // times, slot by slot
-  const bool sph = s->field.spherical != 0;
   int rc = SIM_OK;
   if (!sph && s->sym) {
     // a symmetric plan larger than its buffers: this chunk runs the per-pair kernel
@@ -979,12 +986,12 @@ int run_chunk(sim_t* s) {
   // PLAIN splits tiles too: one event alone must still spread over the SMs
   if (!sph && !s->sym && !team) rc = upload_units(s, true, multi);
   if (rc) return rc;
-  const int gi = sph ? 2 * variant_count() : 2 * s->variant + (multi ? 1 : 0);
+  const int gi = 2 * s->variant + (multi ? 1 : 0);
   const int nl = (multi || sph || team) ? 1 : K;  // step-kernel launches in the chunk
   CK(cudaEventRecord(s->ev0, s->stream));
-  // (the team kernel's grid and shared memory follow the running events: it is
-  // launched directly)
-  if (!plain && !team && !s->opt.disable_graphs) {
+  // (the grids of the team and the spherical kernel follow the running events:
+  // they are launched directly)
+  if (!plain && !team && !sph && !s->opt.disable_graphs) {
     cudaGraphExec_t& graph = s->graphs[gi];
     if (!graph || s->graph_K[gi] != K) {
       if (graph) {
@@ -1510,8 +1517,8 @@ int sim_init(const sim_sensor_t* sensor, const sim_field_t* field, const sim_mob
     }
     s->own_stream = true;
   }
-  s->graphs.assign(2 * variant_count() + 1, nullptr);
-  s->graph_K.assign(2 * variant_count() + 1, -1);
+  s->graphs.assign(2 * variant_count(), nullptr);
+  s->graph_K.assign(2 * variant_count(), -1);
   s->occ_cache.assign(variant_count(), 0);
   s->variant = -1;
   rc = alloc_all(s);

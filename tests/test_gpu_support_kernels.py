@@ -75,3 +75,20 @@ def test_binning_near_pixel_edges(pitch, grid):
     ref = np.zeros((grid, grid), dtype=np.int64)
     np.add.at(ref, (iy[on].astype(int), ix[on].astype(int)), 1)
     assert np.array_equal(pix, ref) and out == (~on).sum()
+
+
+def test_spherical_width_follows_the_running_events():
+    # 40 events: two CTAs each while all run, four once few are left; the
+    # same results as with one CTA throughout
+    name = "plain_3keV_100um"
+    p = W.preset(name)
+    evs = W.make_events(name, n=40, first_id=10)
+    outs = []
+    for opt in ({}, dict(sph_cluster=1)):
+        with cts.Simulator(p["sensor"], p["mobility"], W.field_switches(spherical=1),
+                           keep_final_xy=1, **opt) as sim:
+            outs.append(sim.run(evs, keep_xy_capacity=829))
+            assert (sim.stats()["sph_cluster"] == 1) == bool(opt)
+    for a, b in zip(*outs):
+        assert a["n_steps"] == b["n_steps"] and np.array_equal(a["pixels"], b["pixels"])
+        assert np.array_equal(a["final_xy"], b["final_xy"])
