@@ -2823,31 +2823,157 @@ __device__ __forceinline__ float ggd_variate(uint64_t seed, uint64_t ev, uint32_
   return (b.y >> 31) ? -m : m;
 }
 
+// What a carrier's pixel needs is not the variate but the side of each pixel
+// edge it falls on.  The fast path below computes the variate with the
+// hardware's approximate log2, exp2, cos and rsqrt, together with a bound on
+// how far the FP32 result of ggd_variate can be from it, and decides what that
+// bound decides: a first attempt clearly accepted, a pixel clearly inside its
+// edges.  Everything else (a rejected attempt, or a carrier within about 1e-4
+// of a pixel of an edge) goes to ggd_variate itself, so the counts are
+// those of ggd_variate for every carrier.
+//
+// Error bounds: uniforms have 24 bits.  r^2 = -2 ln u >= 0.01 has an absolute
+// error below 3.4e-7 (log2: 2^-22 on [0.5, 2], 2 ulp outside), the cosine
+// below 6e-7 on [-pi, pi], so |dz| < 1e-5 for |z| < 5.8.  With
+// d = 1/beta + 2/3 <= 4 and v1 >= 0.05 the acceptance test's right side moves
+// by less than 68 |dz| < 7e-4 (its derivative is z - sqrt(d) (v1^2 - 1/v1)):
+// decided beyond 1e-3.  m = alpha U (d v)^(1/beta) then has a relative error
+// below (2e-5 / v1 + 1e-5) / beta + 1e-5, FP32 rounding of ggd_variate
+// included, unless its U^beta comes near underflow.
+struct GgdFast {
+  float alpha, beta, ibeta, d, c, log2_d;
+};
+
+// One attempt from the words w: 1 accepted, 0 rejected, -1 not decided.
+__device__ __forceinline__ int ggd_attempt(const GgdFast& G, uint4 w, float& v1) {
+  const float r2 = -1.38629436f * __log2f(uniform_f(w.x));
+  const float z = -(r2 * rsqrt_approx(r2)) * __cosf(6.28318531f * (uniform_f(w.y) - 0.5f));
+  v1 = fmaf(G.c, z, 1.0f);
+  const float v = v1 * v1 * v1;
+  const float rhs = fmaf(0.5f * z, z, G.d - G.d * v) + G.d * (2.07944154f * __log2f(v1));
+  const float lhs = 0.693147181f * __log2f(uniform_f(w.z));
+  if (!(r2 >= 0.01f)) return -1;
+  if (!(v1 >= 0.05f)) return v1 < -1e-3f ? 0 : -1;
+  return lhs + 1e-3f < rhs ? 1 : lhs - 1e-3f > rhs ? 0 : -1;
+}
+
+// The pixel coordinate floor(x / pitch + half) of an accepted attempt with
+// boost words b: 1 when it is sure (in *px; -1: off the grid), else 0.
+__device__ __forceinline__ int ggd_pixel(const GgdFast& G, float v1, uint4 b, float x0,
+                                         float inv_pitch, float half, int grid_n, int* px) {
+  const float u = uniform_f(b.x);
+  const float t2 = fmaf(3.0f, __log2f(v1), G.log2_d);  // log2 of the gamma variate
+  const float m = G.alpha * u * exp2f(t2 * G.ibeta);
+  const float rel = G.ibeta * (__fdividef(2e-5f, v1) + 1e-5f) + 1e-5f;
+  const float t = fmaf((b.y >> 31) ? x0 - m : x0 + m, inv_pitch, half);
+  const float guard = fmaf(m * inv_pitch, rel, 1e-5f * (1.0f + fabsf(t)));
+  const float f = floorf(t), n = (float)grid_n;
+  // t2 + beta log2(u) >= -100: U^beta and its product stay normal in FP32
+  const bool normal = fmaf(G.beta, __log2f(u), t2) > -100.0f && m < 1e30f;
+  const bool inside = t - f > guard && f + 1.0f - t > guard;  // false for NaN
+  const bool out = t + guard < 0.0f || t - guard >= n;
+  *px = (out || f < 0.0f || f >= n) ? -1 : (int)f;
+  return normal && (inside || out);
+}
+
+__device__ __forceinline__ void generate_count(int px, int py, int grid_n, int* hist, int& lost) {
+  if (px < 0 || py < 0) ++lost;
+  else atomicAdd(&hist[py * grid_n + px], 1);
+}
+
+// One CTA per event.  Bound: integer and FP32 issue of four Philox blocks per
+// carrier.  Each warp takes 32 carriers at a time through the fast path and
+// collects those it does not decide (about one in ten: rejections) in a queue
+// of its own; 32 of them at a time then run further attempts, again through
+// the fast path, and the few that stay undecided call ggd_variate, so that a
+// warp does not wait for its one rejected lane.
 __global__ void __launch_bounds__(256) generate_kernel(const GenEvent* __restrict__ evs,
                                                        double pitch_um, int grid_n,
                                                        int32_t* pixels,
                                                        unsigned long long* outside) {
   __shared__ int hist[kReadoutMaxGrid * kReadoutMaxGrid];
   __shared__ int out_count;
+  __shared__ int queue[8][64];
   const GenEvent e = evs[blockIdx.x];
   const int np = grid_n * grid_n;
   for (int p = threadIdx.x; p < np; p += blockDim.x) hist[p] = 0;
   if (threadIdx.x == 0) out_count = 0;
   __syncthreads();
-  const float a = (float)e.alpha, be = (float)e.beta;
+  const float a = (float)e.alpha, be = (float)e.beta, x0 = (float)e.x0, y0 = (float)e.y0;
   const float inv_pitch = (float)(1.0 / pitch_um), half = 0.5f * (float)grid_n;
+  GgdFast G;
+  G.alpha = a;
+  G.beta = be;
+  G.ibeta = 1.0f / be;
+  G.d = G.ibeta + 1.0f - 1.0f / 3.0f;
+  G.c = rsqrtf(9.0f * G.d);
+  G.log2_d = log2f(G.d);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int* mine = queue[warp];
+  int waiting = 0;  // carriers in the warp's queue (the same in every lane)
   int lost = 0;
-  for (int c = threadIdx.x; c < e.n_pairs; c += blockDim.x) {
-    const float x = (float)e.x0 + ggd_variate(e.seed, e.id, (uint32_t)c, 0u, a, be);
-    const float y = (float)e.y0 + ggd_variate(e.seed, e.id, (uint32_t)c, 1u, a, be);
-    const float fx = floorf(x * inv_pitch + half), fy = floorf(y * inv_pitch + half);
-    if (fx < 0.0f || fy < 0.0f || fx >= (float)grid_n || fy >= (float)grid_n) {
-      ++lost;
-      continue;
+  // 32 (or, at the end, fewer) queued carriers: attempts 1, 2, ... after a
+  // sure rejection, else ggd_variate
+  auto drain = [&](int n) {
+    if (lane < n) {
+      const uint32_t c = (uint32_t)mine[lane];
+      int p[2];
+      bool both = true;
+#pragma unroll
+      for (int axis = 0; axis < 2; ++axis) {
+        int sure = 0;
+        float v1 = 0.0f;
+        for (uint32_t k = 0; k < 4 && sure == 0; ++k)
+          sure = ggd_attempt(
+              G, stream_words(e.seed, e.id, 4u, c, 4u * k + 2u * (uint32_t)axis), v1);
+        both = both && sure == 1 &&
+               ggd_pixel(G, v1, stream_words(e.seed, e.id, 4u, c, 256u + (uint32_t)axis),
+                         axis ? y0 : x0, inv_pitch, half, grid_n, &p[axis]);
+      }
+      if (!both) {
+        // each rounding written out: a pixel edge must not depend on contraction
+        const float x = __fadd_rn(x0, ggd_variate(e.seed, e.id, c, 0u, a, be));
+        const float y = __fadd_rn(y0, ggd_variate(e.seed, e.id, c, 1u, a, be));
+        const float fx = floorf(__fadd_rn(__fmul_rn(x, inv_pitch), half));
+        const float fy = floorf(__fadd_rn(__fmul_rn(y, inv_pitch), half));
+        const bool off = fx < 0.0f || fy < 0.0f || fx >= (float)grid_n || fy >= (float)grid_n;
+        p[0] = off ? -1 : (int)fx;
+        p[1] = off ? -1 : (int)fy;
+      }
+      generate_count(p[0], p[1], grid_n, hist, lost);
     }
-    atomicAdd(&hist[(int)fy * grid_n + (int)fx], 1);
+    __syncwarp();
+  };
+  for (int c0 = warp * 32; c0 < e.n_pairs; c0 += blockDim.x) {
+    const int c = c0 + lane;
+    bool again = false;
+    if (c < e.n_pairs) {
+      float vx, vy;
+      int px = -1, py = -1;
+      const int ax = ggd_attempt(G, stream_words(e.seed, e.id, 4u, (uint32_t)c, 0u), vx);
+      const int ay = ggd_attempt(G, stream_words(e.seed, e.id, 4u, (uint32_t)c, 2u), vy);
+      const int sx = ggd_pixel(G, vx, stream_words(e.seed, e.id, 4u, (uint32_t)c, 256u), x0,
+                               inv_pitch, half, grid_n, &px);
+      const int sy = ggd_pixel(G, vy, stream_words(e.seed, e.id, 4u, (uint32_t)c, 257u), y0,
+                               inv_pitch, half, grid_n, &py);
+      again = ax != 1 || ay != 1 || !sx || !sy;
+      if (!again) generate_count(px, py, grid_n, hist, lost);
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, again);
+    if (again) mine[waiting + __popc(m & ((1u << lane) - 1u))] = c;
+    waiting += __popc(m);
+    __syncwarp();
+    if (waiting >= 32) {
+      waiting -= 32;
+      // the last 32 entries first; the rest stays in place
+      mine += waiting;
+      drain(32);
+      mine -= waiting;
+    }
   }
-  if (lost) atomicAdd(&out_count, lost);
+  drain(waiting);
+  lost = __reduce_add_sync(0xffffffffu, lost);
+  if (lane == 0 && lost) atomicAdd(&out_count, lost);
   __syncthreads();
   for (int p = threadIdx.x; p < np; p += blockDim.x)
     pixels[(int64_t)blockIdx.x * np + p] = hist[p];
