@@ -250,7 +250,8 @@ struct StepArgs {
   int32_t S;                 // slot count
   int32_t fused;             // 1: update positions; 0: write field_out
   double* induced;           // [K][S]: charge induced at each chunk step (e); NULL = off
-  double* induced_px;        // [K][S][9]: the same per pixel of the 3 x 3 window; NULL = off
+  long long* induced_px;     // [K][S][9]: the same per pixel of the 3 x 3 window, in units of
+                             // 2^-44 e; NULL = off
   SymArgs sym;               // the symmetric kernel's plan and buffers
 };
 

@@ -370,7 +370,12 @@ __device__ __forceinline__ bool unit_in_arena(const StepArgs& a, const Unit& U) 
 // expansion z (c3 + c5 (3 <r^2> - 2 z^2)), <r^2> the mean square lateral
 // distance to the pixel's area.  On the collecting surface a pixel's
 // potential is 1 where the readout puts the point, on the back surface 0.
-// FP32 (the offsets from FP64 positions).  Not inlined: every position goes
+// FP32 (the offset from the window's corner from FP64 positions).  An image
+// whose corner terms all have |u v| < zeta^2 / 10 sums them by the arctangent's
+// power series (to t^7, t = u v / (|zeta| r): the next term is below 1e-10), ten
+// operations instead of a square root and an atan2: in a sensor thick against
+// the pixels that is every image but, near the surface, the carrier's own.  FP64
+// operations (two lanes per clock and SM) are kept to three.  Not inlined: every position goes
 // through the same code, so a carrier's potential at the end of a step equals
 // the one at the start of the next bit for bit and the signals telescope.
 __device__ __noinline__ void window_potentials(double x, double y, double z, double wx0,
@@ -388,24 +393,36 @@ __device__ __noinline__ void window_potentials(double x, double y, double z, dou
     return;
   }
   float u[4], v[4];
+  const float pf = (float)pitch;
+  u[0] = (float)(wx0 - x);
+  v[0] = (float)(wy0 - y);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    u[i] = (float)(wx0 + (double)i * pitch - x);
-    v[i] = (float)(wy0 + (double)i * pitch - y);
+  for (int i = 1; i < 4; ++i) {
+    u[i] = fmaf((float)i, pf, u[0]);
+    v[i] = fmaf((float)i, pf, v[0]);
   }
   float acc[9];
 #pragma unroll
   for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
   const float zf = (float)z, h2 = (float)(2.0 * H);
+  const float uv = fmaxf(fabsf(u[0]), fabsf(u[3])) * fmaxf(fabsf(v[0]), fabsf(v[3]));
   for (int n = -M; n <= M; ++n) {
     const float zeta = fmaf((float)n, h2, zf);
     const float az = fabsf(zeta), sg = zeta < 0.0f ? -1.0f : 1.0f, z2 = zeta * zeta;
+    const bool far = uv < 0.1f * z2;
+    const float inv = 1.0f / zeta;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const float r = sqrtf(fmaf(u[i], u[i], fmaf(v[j], v[j], z2)));
-        const float f = sg * atan2f(u[i] * v[j], az * r);
+        const float r2 = fmaf(u[i], u[i], fmaf(v[j], v[j], z2));
+        float f;
+        if (far) {
+          const float t = u[i] * v[j] * inv * rsqrtf(r2), t2 = t * t;
+          f = t * fmaf(t2, fmaf(t2, fmaf(t2, -1.0f / 7.0f, 0.2f), -1.0f / 3.0f), 1.0f);
+        } else {
+          f = sg * atan2f(u[i] * v[j], az * sqrtf(r2));
+        }
         // corner (i, j) is the upper-right corner of pixel (i-1, j-1), the
         // upper-left of (i, j-1), the lower-right of (i-1, j), the lower-left of (i, j)
         if (i >= 1 && j >= 1) acc[(j - 1) * 3 + (i - 1)] += f;
@@ -415,13 +432,12 @@ __device__ __noinline__ void window_potentials(double x, double y, double z, dou
       }
     }
   }
-  const float inv2pi = 0.159154943091895336f, q2 = (float)(pitch * pitch / 6.0);
+  const float inv2pi = 0.159154943091895336f, q2 = pf * pf * (1.0f / 6.0f);
 #pragma unroll
   for (int b = 0; b < 3; ++b) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const float cx = (float)(wx0 + ((double)a + 0.5) * pitch - x);
-      const float cy = (float)(wy0 + ((double)b + 0.5) * pitch - y);
+      const float cx = 0.5f * (u[a] + u[a + 1]), cy = 0.5f * (v[b] + v[b + 1]);
       const float r2 = fmaf(cx, cx, fmaf(cy, cy, q2));
       w[b * 3 + a] = fmaf(acc[b * 3 + a], inv2pi, zf * fmaf(c5, fmaf(3.0f, r2, -2.0f * zf * zf), c3));
     }
@@ -461,6 +477,13 @@ __device__ __forceinline__ int move_carrier(const Phys& ph, int spec, float3 n, 
   return retire;
 }
 
+// A potential (0 .. 1) in units of 2^-44: the pixels' charges are summed as
+// whole numbers, exactly and in any order (FP64 sums of nine pixels took most
+// of a step), up to 5e5 carriers.
+__device__ __forceinline__ long long potential_units(float w) {
+  return __float2ll_rn(w * 17592186044416.0f);
+}
+
 // H times the charge (units of e) that a move from (x0, y0, z0) to (x, y, z)
 // induces on the collecting surface (Shockley-Ramo, weighting potential
 // 1 - z/H, the end point held on [0, H]), or 0 when it is not recorded.
@@ -469,7 +492,7 @@ __device__ __forceinline__ int move_carrier(const Phys& ph, int spec, float3 n, 
 template <int IND>
 __device__ __forceinline__ double induced_charge(const StepArgs& a, int spec, double x0, double y0,
                                                  double z0, double x, double y, double z,
-                                                 double* qpx) {
+                                                 long long* qpx) {
   const Phys& ph = a.ph;
   if (IND == 1 && !a.induced) return 0.0;
   const double zb = fmin(fmax(z, 0.0), ph.H);
@@ -480,8 +503,10 @@ __device__ __forceinline__ double induced_charge(const StepArgs& a, int spec, do
     window_potentials(x, y, zb, ph.wp_x0, ph.wp_y0, ph.pitch, ph.grid_n, ph.H, ph.wp_pairs,
                       ph.wp_c3, ph.wp_c5, w1);
 #pragma unroll
-    for (int j = 0; j < 9; ++j)
-      qpx[j] += spec ? (double)w0[j] - (double)w1[j] : (double)w1[j] - (double)w0[j];
+    for (int j = 0; j < 9; ++j) {
+      const long long d = potential_units(w1[j]) - potential_units(w0[j]);
+      qpx[j] += spec ? -d : d;
+    }
   }
   if (!a.induced) return 0.0;
   return spec ? zb - z0 : z0 - zb;
@@ -497,7 +522,7 @@ __device__ __forceinline__ double update_carrier_at(const StepArgs& a, SlotDev* 
                                                   int spec, int64_t idx, int id, int8_t st,
                                                   double x, double y, double z, int step, int p,
                                                   int k, float Ex, float Ey, float Ez, double azn,
-                                                  double* qpx = nullptr,
+                                                  long long* qpx = nullptr,
                                                   bool* retired = nullptr) {
   const Phys& ph = a.ph;
   [[maybe_unused]] float4* __restrict__ shout = a.A.sh[p ^ 1];
@@ -544,7 +569,7 @@ template <int IND, bool SHADOW = true>
 __device__ __forceinline__ double update_carrier(const StepArgs& a, SlotDev* S, int slot, int spec,
                                                int64_t idx, int step, int p, int k, float Ex,
                                                float Ey, float Ez, double azn,
-                                               double* qpx = nullptr) {
+                                               long long* qpx = nullptr) {
 #ifdef CTS_BOUNDS_CHECK
   if (idx < 0 || idx >= a.A.capacity) {
     atomicOr(a.err, kErrBounds);
@@ -581,14 +606,15 @@ __device__ __forceinline__ void add_induced(const StepArgs& a, int k, int slot, 
 // Adds a warp's per-pixel induced charges (from update_carrier) to the slot's
 // per-step record of the 3 x 3 window (all 32 lanes of the warp call this).
 __device__ __forceinline__ void add_induced_px(const StepArgs& a, int k, int slot,
-                                               const double (&q)[9]) {
+                                               const long long (&q)[9]) {
   if (!a.induced_px) return;
-  double* out = a.induced_px + ((int64_t)k * a.S + slot) * 9;
+  long long* out = a.induced_px + ((int64_t)k * a.S + slot) * 9;
 #pragma unroll
   for (int j = 0; j < 9; ++j) {
-    double v = q[j];
+    long long v = q[j];
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0 && v != 0.0) atomicAdd(out + j, v);
+    if ((threadIdx.x & 31) == 0 && v != 0)
+      atomicAdd(reinterpret_cast<unsigned long long*>(out + j), (unsigned long long)v);
   }
 }
 
@@ -990,7 +1016,7 @@ __global__ void __launch_bounds__(NT, MINB) step_kernel(StepArgs a, int k0, int 
       } else if (a.fused) {
         if constexpr (IND > 0) {
           double q = 0.0;
-          double qpx[9] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+          long long qpx[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
 #pragma unroll
           for (int r = 0; r < R; ++r) {
             const int li = r * NT + tid;
@@ -1283,7 +1309,7 @@ __device__ void sym_tile_update(const StepArgs& a, int gt, int k, int k_end, int
     fz[h] = tz - uz;
   }
   [[maybe_unused]] double q = 0.0;
-  [[maybe_unused]] double qpx[9] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  [[maybe_unused]] long long qpx[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int c = lane + 32 * h;
@@ -1934,7 +1960,7 @@ __global__ void __launch_bounds__(kTeamThreads, 1) team_kernel(StepArgs a, const
       Ez *= ph.f_kc;
     };
     [[maybe_unused]] double qi = 0.0;
-    [[maybe_unused]] double qpx[9] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    [[maybe_unused]] long long qpx[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     // the carrier's move; false once it has left
     auto advance = [&](int spec, int64_t idx, int id, float3 nrm, int c, double& x, double& y,
                        double& z) {
@@ -2041,7 +2067,7 @@ __global__ void update_kernel(StepArgs a, int k, const int32_t* slot_list, int n
     const int n = S->n_h + S->n_e;
     const int64_t cap = a.A.capacity;
     double qi = 0.0;
-    double qpx[9] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    long long qpx[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
       const int spec = t < S->n_h ? 0 : 1;
       const int64_t idx = S->base + (spec ? S->cap_h + (t - S->n_h) : t);
@@ -2690,7 +2716,7 @@ __global__ void __launch_bounds__(1024, 1) spherical_kernel(StepArgs a, const in
     const float kcf = ph.f_kc;
     const double azn = s_azn;
     double qi = 0.0;
-    double qpx[9] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    long long qpx[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     if (!fallback) {
       // each bin's keys (the order within a bin does not matter: a hole
       // counts the smaller keys of its bin)

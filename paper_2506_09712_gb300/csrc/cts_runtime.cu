@@ -73,7 +73,11 @@ constexpr int kSymVariantPlain = 0;  // sym_nt384_r8_warp
 // requests behind whatever else its process runs on the GPU (and the events of
 // a stream are meant to overlap: alone, an 8 keV event of a served stream
 // takes 8.7 ms with teams, 26 ms without).
+// With pixel signals the line lies at twice as much: the potentials of a tile's
+// 512 carriers are one CTA's work in the per-pair kernel (eight events of 3000
+// carriers: 38.7 -> 92.1 us a step with them, the team kernel 40.3 -> 50.4).
 constexpr double kTeamMaxLoad = 2.4e4;
+constexpr double kTeamMaxLoadPixels = 4.8e4;
 // a team's CTAs have at least this many rows of kTeamRow carriers each (the
 // step of an 829-carrier event no longer shortens beyond 52 CTAs)
 constexpr int kTeamMinRows = 4;
@@ -123,7 +127,7 @@ struct HostSlot {
   std::vector<double> induced;  // per executed step (options.keep_induced)
   double induced_q = 0.0;
   std::vector<double> induced_px;  // [step][9] per executed step
-  double induced_pxq[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+  long long induced_pxq[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};  // units of 2^-44 e
 };
 
 }  // namespace
@@ -159,8 +163,9 @@ struct sim_t {
   float* d_drift = nullptr;           // sampled drift field (optional)
   double* d_induced = nullptr;        // [K][S] induced charge per chunk step (keep_induced)
   double* h_induced = nullptr;
-  double* d_induced_px = nullptr;     // [K][S][9] the same per pixel of the 3 x 3 window
-  double* h_induced_px = nullptr;
+  // [K][S][9] the same per pixel of the 3 x 3 window, in units of 2^-44 e
+  long long* d_induced_px = nullptr;
+  long long* h_induced_px = nullptr;
   std::vector<double> drift_host;     // the caller's samples, copied at init
   int32_t* d_err = nullptr;
   float* d_field = nullptr;
@@ -858,7 +863,7 @@ int issue_chunk(sim_t* s, int K, bool multi) {
   if (s->d_induced)
     CK(cudaMemsetAsync(s->d_induced, 0, (size_t)K * s->S * sizeof(double), s->stream));
   if (s->d_induced_px)
-    CK(cudaMemsetAsync(s->d_induced_px, 0, (size_t)K * s->S * 9 * sizeof(double), s->stream));
+    CK(cudaMemsetAsync(s->d_induced_px, 0, (size_t)K * s->S * 9 * sizeof(long long), s->stream));
   if (s->field.spherical) {
     // the spherical model: one cluster of CTAs per slot runs all K steps of
     // its event
@@ -908,7 +913,7 @@ int issue_chunk(sim_t* s, int K, bool multi) {
   CK(d2h(s, s->h_summary, s->d_summary, s->S * sizeof(SlotSummary)));
   if (s->d_induced) CK(d2h(s, s->h_induced, s->d_induced, (size_t)K * s->S * sizeof(double)));
   if (s->d_induced_px)
-    CK(d2h(s, s->h_induced_px, s->d_induced_px, (size_t)K * s->S * 9 * sizeof(double)));
+    CK(d2h(s, s->h_induced_px, s->d_induced_px, (size_t)K * s->S * 9 * sizeof(long long)));
   CK(d2h(s, s->h_err, s->d_err, sizeof(int32_t)));
   return SIM_OK;
 }
@@ -962,7 +967,7 @@ int run_chunk(sim_t* s) {
     const bool full = W >= (serve ? kSymMinWorkServe : kSymMinWork);
     int rcv = set_variant(s, full ? sym_v : kPairVariant);
     if (rcv) return rcv;
-    if (!serve && W < kTeamMaxLoad * max_n && !full && !s->field.spherical &&
+    if (!serve && W < (s->d_induced_px ? kTeamMaxLoadPixels : kTeamMaxLoad) * max_n && !full && !s->field.spherical &&
         !s->opt.step_launches) {
       rcv = plan_team(s, &team);
       if (rcv) return rcv;
@@ -1178,7 +1183,7 @@ int pump(sim_t* s, bool defer, bool* progressed) {
         if (s->h_induced_px)
           for (int j = 0; j < 9; ++j) {
             h.induced_pxq[j] += s->h_induced_px[(kk * s->S + k) * 9 + j];
-            h.induced_px.push_back(h.induced_pxq[j]);
+            h.induced_px.push_back((double)h.induced_pxq[j] * 0x1p-44);
           }
       }
     }
