@@ -3008,84 +3008,144 @@ __global__ void __launch_bounds__(256) generate_kernel(const GenEvent* __restric
 
 // ---------------------------------------------------------------------------
 // Detector readout of pixel-count maps (Sec. 4.1 selection, Sec. 4.2 noise):
-// one CTA per event.  Pixel energies with Gaussian noise from the event's
-// stream (purpose 3, carrier = pixel), the centre at the largest pixel (first
-// in row-major order on ties), the 3 x 3 cluster, the 7 x 7 pile-up veto and
-// the cluster-energy window; accepted clusters add their on-grid pixels to
-// the single-pixel spectrum.
+// pixel energies with Gaussian noise from the event's stream (purpose 3,
+// carrier = pixel), the centre at the largest pixel (first in row-major order
+// on ties), the 3 x 3 cluster, the 7 x 7 pile-up veto and the cluster-energy
+// window; accepted clusters add their on-grid pixels to the single-pixel
+// spectrum.
+//
+// Bound: FP64 arithmetic (a logarithm, a square root and a cosine per pixel at
+// two FP64 lanes per clock and SM).  Only the nine pixels of a cluster are
+// reported, the others are compared: with the largest pixel, and with the veto
+// threshold.  So every pixel is first computed in FP32, and in FP64 (the value
+// all decisions are defined by) where it is reported, where FP32 leaves more
+// than one candidate for the largest, where it lies within FP32's error of the
+// threshold, and everywhere when the energies themselves are asked for.  A CTA
+// takes several events, so that the clusters' FP64 pixels fill its threads.
+// 20000 maps of 9 x 9: 583 us with every pixel in FP64.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) readout_kernel(ReadoutArgs r) {
-  __shared__ double e[kReadoutMaxGrid * kReadoutMaxGrid];
-  __shared__ double wv[8];
-  __shared__ int wi[8];
-  const int ev = blockIdx.x, n = r.grid_n, np = n * n;
-  const int32_t* cnt = r.counts + (int64_t)ev * np;
-  const uint64_t seed = r.seeds[ev], id = r.ids[ev];
-  double best = -INFINITY;
-  int bi = np;
-  for (int p = threadIdx.x; p < np; p += blockDim.x) {
-    double g = 0.0;
-    if (r.noise_keV > 0.0) g = normals_d(stream_words(seed, id, 3u, (uint32_t)p, 0u)).x;
-    const double v = (double)cnt[p] * r.ev_per_pair * 1e-3 + r.noise_keV * g;
-    e[p] = v;
-    if (r.pixel_keV) r.pixel_keV[(int64_t)ev * np + p] = v;
-    if (v > best || (v == best && p < bi)) {
-      best = v;
-      bi = p;
-    }
-  }
-  // (largest energy, smallest index) over the block
-  for (int o = 16; o > 0; o >>= 1) {
-    const double ov = __shfl_down_sync(0xffffffffu, best, o);
-    const int oi = __shfl_down_sync(0xffffffffu, bi, o);
-    if (ov > best || (ov == best && oi < bi)) {
-      best = ov;
-      bi = oi;
-    }
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) {
-    wv[warp] = best;
-    wi[warp] = bi;
+constexpr int kReadoutThreads = 256;
+constexpr int kReadoutEvents = 28;       // 9 x 28 cluster pixels: one round of threads
+constexpr int kReadoutPixels = 8192;     // FP32 energies in shared memory
+
+__device__ __forceinline__ double readout_energy(const ReadoutArgs& r, uint64_t seed, uint64_t id,
+                                                 int p, int count) {
+  double g = 0.0;
+  if (r.noise_keV > 0.0) g = normals_d(stream_words(seed, id, 3u, (uint32_t)p, 0u)).x;
+  return (double)count * r.ev_per_pair * 1e-3 + r.noise_keV * g;
+}
+
+__global__ void __launch_bounds__(kReadoutThreads) readout_kernel(ReadoutArgs r, int n_events,
+                                                                  int per) {
+  __shared__ float ef[kReadoutPixels];
+  __shared__ double ec[kReadoutEvents][9];
+  __shared__ int centre[kReadoutEvents], veto[kReadoutEvents];
+  const int n = r.grid_n, np = n * n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ev0 = blockIdx.x * per, ne = min(per, n_events - ev0);
+  const int32_t* cnt = r.counts + (int64_t)ev0 * np;
+  const float wf = (float)(r.ev_per_pair * 1e-3), nf = (float)r.noise_keV;
+  // FP32 against FP64: the conversions and the product (2^-22 of the count's
+  // energy), the normal (|g| < 5.8, below 4e-6 off) and the sum
+  auto slack = [&](float v) { return 1e-6f * fabsf(v) + 2e-5f * nf; };
+  for (int e = tid; e < ne; e += kReadoutThreads) veto[e] = 0;
+  for (int q = tid; q < ne * np; q += kReadoutThreads) {
+    const int e = q / np, p = q - e * np;
+    float g = 0.0f;
+    if (r.noise_keV > 0.0)
+      g = normals_f(stream_words(r.seeds[ev0 + e], r.ids[ev0 + e], 3u, (uint32_t)p, 0u)).x;
+    ef[q] = fmaf(nf, g, (float)cnt[q] * wf);
+    if (r.pixel_keV)
+      r.pixel_keV[(int64_t)ev0 * np + q] =
+          readout_energy(r, r.seeds[ev0 + e], r.ids[ev0 + e], p, cnt[q]);
   }
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-    if (wv[w] > best || (wv[w] == best && wi[w] < bi)) {
-      best = wv[w];
-      bi = wi[w];
+  // the largest pixel: a warp per event
+  for (int e = warp; e < ne; e += kReadoutThreads / 32) {
+    const float* v = ef + e * np;
+    float top = -INFINITY;
+    for (int p = lane; p < np; p += 32) top = fmaxf(top, v[p]);
+    for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+    const float edge = top - 2.0f * slack(top);
+    int close = 0, bi = np;
+    for (int p = lane; p < np; p += 32)
+      if (!(v[p] < edge)) {
+        ++close;
+        bi = min(bi, p);
+      }
+    if (__reduce_add_sync(0xffffffffu, close) > 1) {
+      // several candidates (two nearly equal pixels, or no noise): by FP64
+      double best = -INFINITY;
+      bi = np;
+      for (int p = lane; p < np; p += 32)
+        if (!(v[p] < edge)) {
+          const double x =
+              readout_energy(r, r.seeds[ev0 + e], r.ids[ev0 + e], p, cnt[e * np + p]);
+          if (x > best) {
+            best = x;
+            bi = p;
+          }
+        }
+      for (int o = 16; o > 0; o >>= 1) {
+        const double ox = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (ox > best || (ox == best && oi < bi)) {
+          best = ox;
+          bi = oi;
+        }
+      }
+    } else {
+      bi = __reduce_min_sync(0xffffffffu, bi);
     }
-  const int bx = bi % n, by = bi / n;
-  ClusterRec c;
-  c.e_cluster = 0.0;
-  for (int dy = -1; dy <= 1; ++dy)
-    for (int dx = -1; dx <= 1; ++dx) {
-      const int x = bx + dx, y = by + dy;
-      const bool on = x >= 0 && y >= 0 && x < n && y < n;
-      const double v = on ? e[y * n + x] : __longlong_as_double(0x7ff8000000000000ll);
-      c.e[(dy + 1) * 3 + (dx + 1)] = v;
-      if (on) c.e_cluster += v;
-    }
-  int veto = 0;
-  for (int dy = -3; dy <= 3; ++dy)
-    for (int dx = -3; dx <= 3; ++dx) {
-      if (dx >= -1 && dx <= 1 && dy >= -1 && dy <= 1) continue;
-      const int x = bx + dx, y = by + dy;
-      if (x < 0 || y < 0 || x >= n || y >= n) continue;
-      if (e[y * n + x] > r.veto_factor * r.noise_keV) veto = 1;
-    }
-  c.cx = bx;
-  c.cy = by;
-  c.vetoed = veto;
-  c.accepted = !veto && fabs(c.e_cluster - r.beam_keV) <= r.window_keV;
-  r.clusters[ev] = c;
-  if (c.accepted && r.spectrum)
+    if (lane == 0) centre[e] = bi;
+  }
+  __syncthreads();
+  // the clusters' pixels in FP64, off-grid ones NaN
+  for (int q = tid; q < ne * 9; q += kReadoutThreads) {
+    const int e = q / 9, k = q - 9 * e;
+    const int x = centre[e] % n + k % 3 - 1, y = centre[e] / n + k / 3 - 1;
+    const bool on = x >= 0 && y >= 0 && x < n && y < n;
+    ec[e][k] = on ? readout_energy(r, r.seeds[ev0 + e], r.ids[ev0 + e], y * n + x,
+                                   cnt[e * np + y * n + x])
+                  : __longlong_as_double(0x7ff8000000000000ll);
+  }
+  // the ring around them against the veto threshold
+  const double limit = r.veto_factor * r.noise_keV;
+  const float lf = (float)limit;
+  for (int q = tid; q < ne * 49; q += kReadoutThreads) {
+    const int e = q / 49, k = q - 49 * e, dx = k % 7 - 3, dy = k / 7 - 3;
+    if (dx >= -1 && dx <= 1 && dy >= -1 && dy <= 1) continue;
+    const int x = centre[e] % n + dx, y = centre[e] / n + dy;
+    if (x < 0 || y < 0 || x >= n || y >= n) continue;
+    const float v = ef[e * np + y * n + x];
+    const float off = slack(v) + 1e-6f * fabsf(lf);
+    bool over = v > lf;
+    if (!(fabsf(v - lf) > off))
+      over = readout_energy(r, r.seeds[ev0 + e], r.ids[ev0 + e], y * n + x,
+                            cnt[e * np + y * n + x]) > limit;
+    if (over) veto[e] = 1;
+  }
+  __syncthreads();
+  for (int e = tid; e < ne; e += kReadoutThreads) {
+    ClusterRec c;
+    c.e_cluster = 0.0;
+#pragma unroll
     for (int k = 0; k < 9; ++k) {
-      const double v = c.e[k];
-      if (isnan(v)) continue;
-      const double b = floor((v - r.spec_lo_keV) / r.spec_bin_keV);
-      if (b >= 0.0 && b < (double)r.n_bins) atomicAdd(r.spectrum + (int64_t)b, 1ull);
+      c.e[k] = ec[e][k];
+      if (!isnan(c.e[k])) c.e_cluster += c.e[k];
     }
+    c.cx = centre[e] % n;
+    c.cy = centre[e] / n;
+    c.vetoed = veto[e];
+    c.accepted = !c.vetoed && fabs(c.e_cluster - r.beam_keV) <= r.window_keV;
+    r.clusters[ev0 + e] = c;
+    if (c.accepted && r.spectrum)
+      for (int k = 0; k < 9; ++k) {
+        const double v = c.e[k];
+        if (isnan(v)) continue;
+        const double b = floor((v - r.spec_lo_keV) / r.spec_bin_keV);
+        if (b >= 0.0 && b < (double)r.n_bins) atomicAdd(r.spectrum + (int64_t)b, 1ull);
+      }
+  }
 }
 
 // FP32 FMA throughput probe: independent FMA chains per thread (packed f32x2
@@ -3371,7 +3431,10 @@ cudaError_t launch_generate(const GenEvent* ev, int n_events, double pitch_um, i
 }
 
 cudaError_t launch_readout(const ReadoutArgs& r, int n_events, cudaStream_t s) {
-  if (n_events > 0) readout_kernel<<<n_events, 256, 0, s>>>(r);
+  if (n_events <= 0) return cudaSuccess;
+  const int np = r.grid_n * r.grid_n;
+  const int per = kReadoutPixels / np < kReadoutEvents ? kReadoutPixels / np : kReadoutEvents;
+  readout_kernel<<<(n_events + per - 1) / per, kReadoutThreads, 0, s>>>(r, n_events, per);
   return cudaGetLastError();
 }
 
