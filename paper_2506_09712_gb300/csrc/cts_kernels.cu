@@ -3432,8 +3432,11 @@ cudaError_t launch_generate(const GenEvent* ev, int n_events, double pitch_um, i
 
 cudaError_t launch_readout(const ReadoutArgs& r, int n_events, cudaStream_t s) {
   if (n_events <= 0) return cudaSuccess;
+  // events per CTA: a round of cluster pixels, what shared memory holds, and
+  // few enough that a small call still has eight CTAs per SM of a 152-SM part
   const int np = r.grid_n * r.grid_n;
-  const int per = kReadoutPixels / np < kReadoutEvents ? kReadoutPixels / np : kReadoutEvents;
+  int per = kReadoutPixels / np < kReadoutEvents ? kReadoutPixels / np : kReadoutEvents;
+  if (n_events / 1216 < per) per = n_events < 1216 ? 1 : n_events / 1216;
   readout_kernel<<<(n_events + per - 1) / per, kReadoutThreads, 0, s>>>(r, n_events, per);
   return cudaGetLastError();
 }
