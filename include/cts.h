@@ -127,11 +127,15 @@ typedef struct sim_options_t {
   int32_t queue_capacity;  /* bound of the admission queue (default 65536) */
   int32_t variant;         /* pair-kernel variant + 1; 0 = default choice: per
                               chunk, the symmetric kernel when the running
-                              events hold at least 4.0e8 carrier pairs (sum
-                              of N^2) -- variant 1 (12 warps per SM), or 13
-                              (8 warps) once an event has more than 640
+                              events hold at least 1.6e8 carrier pairs (sum
+                              of N^2; 4.0e8 if they are smaller than 1536
+                              carriers) -- variant 1 (12 warps per SM), or 13
+                              (8 warps) below 2.6e8 pairs, up to 3072
+                              carriers, and once an event has more than 640
                               tiles of 64 carriers -- the per-pair kernel
-                              (variant 2) below that; SERVE: variant 13 from
+                              (variant 2) below that, and below 2.4e4 times
+                              the largest event's carriers the team kernel (a
+                              team of SMs per event; reported as variant 2); SERVE: variant 13 from
                               2.8e8 pairs, else variant 2; PLAIN: variant 1 */
   int32_t disable_graphs;  /* 1 = launch K-step chunks directly, not as CUDA graphs */
   int32_t keep_final_xy;   /* 1 = keep collected (x, y) and retire steps for poll */

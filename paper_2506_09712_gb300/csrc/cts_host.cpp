@@ -221,19 +221,32 @@ int plan_units(const int32_t* n_h, const int32_t* n_e, int n_slots, int tile_i, 
 // writes one partial field per tile of its blocks and per tile of its J
 // range; a tile's field is the sum of its partials in unit order.
 // ---------------------------------------------------------------------------
-void sym_shape(int ntiles, int* rb, int* rj) {
+void sym_shape(int ntiles, int level, int* rb, int* rj) {
   // small events: short units, so that each step of an event is spread over
   // many warps; large events: fewer, larger units (fewer partial fields)
   if (ntiles <= 160) {
     *rb = 1;
-    *rj = 8;
+    *rj = level ? 4 : 8;
   } else if (ntiles <= 640) {
-    *rb = 2;
-    *rj = 16;
+    *rb = level ? 1 : 2;
+    *rj = level > 1 ? 8 : 16;
   } else {
-    *rb = 8;
+    *rb = 8 >> level;
     *rj = 16;
   }
+}
+
+double sym_units(const int32_t* n_h, const int32_t* n_e, int n_slots, int level) {
+  double units = 0.0;  // about half of a slot's blocks x tiles rectangles
+  for (int s = 0; s < n_slots; ++s) {
+    const int nh = std::max(n_h[s], 0), ne = std::max(n_e[s], 0);
+    if (nh <= 0) continue;
+    const int nt = (nh + kSymPlanTile - 1) / kSymPlanTile + (ne + kSymPlanTile - 1) / kSymPlanTile;
+    int rb, rj;
+    sym_shape(nt, level, &rb, &rj);
+    units += 0.5 * ((double)nt / (kSymPlanTpb * rb)) * ((double)nt / rj);
+  }
+  return units;
 }
 
 namespace {
@@ -241,11 +254,11 @@ namespace {
 // The plan of one slot with th hole tiles and te electron tiles: its pair
 // units longest first (partials numbered from 0), its update units, and the
 // partial lists of its tiles in unit order.
-SymSlotTemplate sym_slot_template(int th, int te) {
+SymSlotTemplate sym_slot_template(int th, int te, int level, int updates) {
   constexpr int B = kSymPlanTpb;
   SymSlotTemplate T;
   int rb, rj;
-  sym_shape(th + te, &rb, &rj);
+  sym_shape(th + te, level, &rb, &rj);
   std::vector<SymUnitPlan> su;
   std::vector<int64_t> work;
   auto rows = [&](int spec_i, int nti, int spec_j, int ntj, bool same) {
@@ -283,9 +296,9 @@ SymSlotTemplate sym_slot_template(int th, int te) {
     T.n_partials += u.jt1 - u.jt0;
     T.pair.push_back(u);
   }
-  // update units: a few tiles each (at most 64 units a slot)
+  // update units: a few tiles each (at most `updates` units a slot)
   const int nt = th + te;
-  const int tu = std::max(kSymPlanUpdateTiles, (nt + 63) / 64);
+  const int tu = std::max(kSymPlanUpdateTiles, (nt + updates - 1) / updates);
   for (int t = 0; t < nt; t += tu)
     T.upd.push_back(SymUnitPlan{0, 0, 0, 0, 0, t, std::min(t + tu, nt), 0, 0, 0, 1,
                                 (int32_t)T.pair.size()});
@@ -313,7 +326,8 @@ SymSlotTemplate sym_slot_template(int th, int te) {
 
 }  // namespace
 
-int plan_sym(const int32_t* n_h, const int32_t* n_e, int n_slots, int max_units, SymPlan* out) {
+int plan_sym(const int32_t* n_h, const int32_t* n_e, int n_slots, int max_units, SymPlan* out,
+             int level, int updates) {
   out->units.clear();
   out->tiles.clear();
   out->lists.clear();
@@ -334,8 +348,10 @@ int plan_sym(const int32_t* n_h, const int32_t* n_e, int n_slots, int max_units,
     const int nh = std::max(n_h[s], 0), ne = std::max(n_e[s], 0);
     if (nh <= 0) continue;  // an event with no hole is finished
     const int th = (nh + T - 1) / T, te = (ne + T - 1) / T;
-    auto it = out->memo.find({th, te});
-    if (it == out->memo.end()) it = out->memo.emplace(std::make_pair(th, te), sym_slot_template(th, te)).first;
+    const std::array<int, 4> key{th, te, level, updates};
+    auto it = out->memo.find(key);
+    if (it == out->memo.end())
+      it = out->memo.emplace(key, sym_slot_template(th, te, level, updates)).first;
     const SymSlotTemplate& st = it->second;
     const int64_t pbase = out->n_partials;
     if (pbase + st.n_partials > INT32_MAX) return -2;

@@ -1,5 +1,6 @@
 // cts_host_impl.h -- C++ interface of the pure host logic (cts_host.cpp).
 #pragma once
+#include <array>
 #include <cstdint>
 #include <map>
 #include <utility>
@@ -33,6 +34,7 @@ int plan_units(const int32_t* n_h, const int32_t* n_e, int n_slots, int tile_i, 
 constexpr int kSymPlanTile = 64;   // carriers per tile
 constexpr int kSymPlanTpb = 4;     // tiles per I block
 constexpr int kSymPlanUpdateTiles = 1;  // tiles per update unit (at least)
+constexpr int kSymPlanUpdates = 64;     // update units a slot at most
 constexpr int kSymPlanUpdateLag = 32;   // slots of pair units before a slot's update units
 struct SymUnitPlan {
   // kind 0: pair unit; kind 1: update unit of the slot's tiles [jt0, jt1)
@@ -58,12 +60,20 @@ struct SymPlan {
   std::vector<int32_t> slot_tile0;    // global index of a slot's first tile (-1: none)
   std::vector<int32_t> slot_ntiles;   // tiles of the slot
   int64_t n_partials = 0;             // partial tiles the units write
-  // slot plans by (th, te), kept across calls on the same SymPlan
-  std::map<std::pair<int, int>, SymSlotTemplate> memo;
+  // slot plans by (th, te, unit level, update units), kept across calls on the
+  // same SymPlan
+  std::map<std::array<int, 4>, SymSlotTemplate> memo;
 };
-// Unit shape (I blocks x J tiles) of a slot with `ntiles` tiles.
-void sym_shape(int ntiles, int* rb, int* rj);
-int plan_sym(const int32_t* n_h, const int32_t* n_e, int n_slots, int max_units, SymPlan* out);
+// Unit shape (I blocks x J tiles) of a slot with `ntiles` tiles: level 0 for a
+// GPU full of work, levels 1 and 2 smaller ones for few events (up to 160
+// tiles: 1 x 8, then 1 x 4).
+constexpr int kSymPlanLevels = 3;
+void sym_shape(int ntiles, int level, int* rb, int* rj);
+// About the pair units the slots have at a level.
+double sym_units(const int32_t* n_h, const int32_t* n_e, int n_slots, int level);
+// updates: the most update units of a slot.
+int plan_sym(const int32_t* n_h, const int32_t* n_e, int n_slots, int max_units, SymPlan* out,
+             int level = 0, int updates = kSymPlanUpdates);
 
 // Fano-distributed carrier-pair count of one photon (see cts_fano_pairs).
 int fano_pairs(uint64_t seed, uint64_t event_id, double energy_keV, double fano);

@@ -38,12 +38,32 @@ constexpr int kDefaultSlots = 256;
 constexpr int kDefaultK = 32;
 constexpr size_t kLaunchLogCap = size_t(1) << 20;
 constexpr int64_t kDefaultBudget = 1ll << 30;
-// Default kernel choice per chunk: the symmetric kernel from this many
-// resident carrier pairs per step (sum of N^2), the per-pair kernel below.
-// Whole 64-event 20 keV batches with the 12-warp symmetric kernel, 32-step
-// chunks: 462 / 458 / 452 / 448 ms with the switch at 1.2e8 / 1.8e8 / 2.8e8
-// / 4.0e8 pairs (about 17 partly collected events)
-constexpr double kSymMinWork = 4.0e8;
+// Default kernel choice per chunk: the symmetric kernel from kSymMinWork
+// resident carrier pairs per step (sum of N^2), the per-pair kernel below.  With
+// few events a step is as long as one event's units and updates one after
+// another, so units of four J tiles take the place of eight until enough
+// events run: below kSymFullWork pairs or kSymFullEvents events.  Below
+// kSymShortWork, and for events of up to kSymShortCarriers (whose blocks leave
+// partly filled units of eight), 8 warps per SM instead of 12.  Events of less
+// than kSymSmallCarriers fill no units: they take the symmetric kernel, with
+// units of eight, only from kSymMinWorkSmall (829 carriers, 250 events 86 in
+// the per-pair kernel, 142 in this one).  An event's size here is the running
+// events' pair-weighted mean, sum of N^2 over sum of N.
+// Microseconds per step (per-pair; 1 x 8 units, 12 warps; 1 x 4, 8 warps;
+// 1 x 4, 12 warps): 5525 carriers, 4 events 58.6; 133.7; 73.4; 91.6, 6 events
+// 77.3; 138.7; 75.4; 92.6, 8 events 97.0; 143.3; 76.1; 95.0, 12 events 136.8;
+// 146.0; 112.6; 101.3, 16 events 179.6; 149.3; 145.8; 143.9, 20 events 220.4;
+// 161.4; 178.9; 165.7, 32 events 353.2; 257.0; 273.7; 264.3.  2210 carriers, 32
+// events 67.6; 108.1; 57.9; 75.4, 128 events 232.5; 255.8; 205.9; 237.2.  Two
+// species of 4000, 4 events 101.5; 146.5; 82.1; 97.0, 10 events 198.9; 182.1;
+// 140.9; 134.1.
+constexpr double kSymMinWork = 1.6e8;
+constexpr double kSymShortWork = 2.6e8;
+constexpr double kSymFullWork = 5.5e8;
+constexpr int kSymFullEvents = 18;
+constexpr double kSymShortCarriers = 3072.0;
+constexpr double kSymSmallCarriers = 1536.0;
+constexpr double kSymMinWorkSmall = 4.0e8;
 // SERVE keeps the 8-warp symmetric kernel and the switch at 2.8e8 pairs: at
 // the moderate occupancy of a served stream (about 27 mixed events at 0.7x
 // saturation) its steps are shorter; the serving mix's p50 / p99 latency at
@@ -83,6 +103,13 @@ constexpr double kTeamMaxLoadPixels = 4.8e4;
 constexpr int kTeamMinRows = 4;
 constexpr int kMaxUnits = 1 << 16;
 constexpr int kMaxSymUnits = 1 << 18;  // units of one step of the symmetric kernel
+// Large events (over 160 tiles): units are halved, once or twice, while a step
+// has fewer than this many per SM, and a slot has up to kSymUpdatesLarge update
+// units.  One 200 keV track's step took 4.9 ms: 2.4 rounds of 8 x 16 units,
+// then 64 update units of 27 tiles one after another; with finer updates 3.5
+// ms, with finer pair units too 3.1 ms (the pairs at 4.2e12/s: 2.9 ms).
+constexpr int kSymUnitsPerSm = 64;
+constexpr int kSymUpdatesLarge = 1024;
 // upload_sym_plan: the plan needs more units or tiles than the buffers hold
 constexpr int kSymPlanTooLarge = 1;
 constexpr int kDefaultQueue = 1 << 16;
@@ -183,6 +210,9 @@ struct sim_t {
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   std::vector<cudaEvent_t> lev;  // per-launch events (time_launches): K + 1
 
+  // unit level and most update units a slot of the symmetric plan: the default
+  // choice of a chunk sets them, everything else plans level 0
+  int sym_level = 0, sym_updates = kSymPlanUpdates;
   // the symmetric kernel's plan of the current chunk and its buffers (the
   // partial fields and lists grow with the plan; growing them drops the
   // captured graphs, which hold their addresses)
@@ -683,7 +713,8 @@ int upload_sym_plan(sim_t* s, const std::vector<SymGeom>& g) {
     ne[k] = g[k].n_e;
   }
   SymPlan& P = s->splan;
-  const int prc = plan_sym(nh.data(), ne.data(), n_slots, kMaxSymUnits, &P);
+  const int prc =
+      plan_sym(nh.data(), ne.data(), n_slots, kMaxSymUnits, &P, s->sym_level, s->sym_updates);
   if (prc == -2 || (prc == 0 && (int64_t)P.tiles.size() > s->sym_tiles_cap)) return kSymPlanTooLarge;
   if (prc != 0) {
     s->err = "symmetric unit plan failed";
@@ -926,6 +957,8 @@ int run_chunk(sim_t* s) {
   const int K = plain ? 1 : s->K;
   bool team = false;
   s->team_grid = 0;
+  s->sym_level = 0;
+  s->sym_updates = kSymPlanUpdates;
   const bool sph = s->field.spherical != 0;
   if (plain || sph) {
     // the update launch walks the running slot listed in d_list, the
@@ -953,18 +986,40 @@ int run_chunk(sim_t* s) {
     // the default choice per chunk: the symmetric kernel while the resident
     // pair work fills the GPU, the per-pair kernel (finer work units, shorter
     // steps) below it; the events' state is the same for both
-    double W = 0.0;
-    int max_tiles = 0, max_n = 0;
+    double W = 0.0, n_sum = 0.0;
+    int max_tiles = 0, max_n = 0, n_run = 0;
     for (auto& h : s->slots)
       if (h.used && h.running) {
         W += (double)(h.n_h + h.n_e) * (double)(h.n_h + h.n_e);
         max_n = std::max(max_n, h.n_h + h.n_e);
+        n_sum += h.n_h + h.n_e;
+        ++n_run;
         max_tiles = std::max(max_tiles, (h.n_h + kSymTile - 1) / kSymTile +
                                             (h.n_e + kSymTile - 1) / kSymTile);
       }
     const bool serve = s->opt.mode == CTS_MODE_SERVE;
-    const int sym_v = (serve || max_tiles > kSymLargeTiles) ? kSymVariantLarge : kSymVariant;
-    const bool full = W >= (serve ? kSymMinWorkServe : kSymMinWork);
+    const double mean_n = n_sum > 0.0 ? W / n_sum : 0.0;
+    const bool full = W >= (serve ? kSymMinWorkServe
+                                  : mean_n < kSymSmallCarriers ? kSymMinWorkSmall : kSymMinWork);
+    const bool large = max_tiles > 160;
+    int sym_v = (serve || max_tiles > kSymLargeTiles) ? kSymVariantLarge : kSymVariant;
+    if (!serve && large) {
+      std::vector<int32_t> nh, ne;
+      for (auto& h : s->slots)
+        if (h.used && h.running) {
+          nh.push_back(h.n_h);
+          ne.push_back(h.n_e);
+        }
+      while (s->sym_level + 1 < kSymPlanLevels &&
+             sym_units(nh.data(), ne.data(), (int)nh.size(), s->sym_level) <
+                 (double)kSymUnitsPerSm * s->sm_count)
+        ++s->sym_level;
+      s->sym_updates = kSymUpdatesLarge;
+    } else if (!serve && mean_n >= kSymSmallCarriers &&
+               (mean_n <= kSymShortCarriers || W < kSymFullWork || n_run < kSymFullEvents)) {
+      s->sym_level = 1;
+      if (mean_n <= kSymShortCarriers || W < kSymShortWork) sym_v = kSymVariantLarge;
+    }
     int rcv = set_variant(s, full ? sym_v : kPairVariant);
     if (rcv) return rcv;
     if (!serve && W < (s->d_induced_px ? kTeamMaxLoadPixels : kTeamMaxLoad) * max_n && !full && !s->field.spherical &&
@@ -979,6 +1034,8 @@ int run_chunk(sim_t* s) {
   if (!sph && s->sym) {
     // a symmetric plan larger than its buffers: this chunk runs the per-pair kernel
     rc = upload_units(s, true, true);
+    s->sym_level = 0;
+    s->sym_updates = kSymPlanUpdates;
     if (rc == kSymPlanTooLarge) {
       rc = set_variant(s, kPairVariant);
       if (rc) return rc;
