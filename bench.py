@@ -259,15 +259,18 @@ def aggregate(dist, device, elapsed_ms: float, *counts: float):
 # ---------------------------------------------------------------------------
 def kernel_source_hash() -> str:
     """Hash of the source the step kernel is compiled from: the data layout
-    (cts_internal.h up to its launcher declarations), the device helpers and
-    the kernel (cts_kernels.cu up to the next kernel) and the variant table.
+    (cts_internal.h up to its launcher declarations), the pair loops
+    (cts_pairs.cuh), the device helpers and the kernel (cts_kernels.cu up to
+    the next kernel) and the variant table.
     Other kernels in the same files do not change it."""
     csrc = os.path.join(ROOT, "paper_2506_09712_gb300", "csrc")
     with open(os.path.join(csrc, "cts_internal.h")) as fh:
         hdr = fh.read()
     with open(os.path.join(csrc, "cts_kernels.cu")) as fh:
         ker = fh.read()
-    parts = [hdr.split("// ---- kernel launchers")[0],
+    with open(os.path.join(csrc, "cts_pairs.cuh")) as fh:
+        loops = fh.read()
+    parts = [hdr.split("// ---- kernel launchers")[0], loops,
              ker.split("// Update alone:")[0],
              ker[ker.index("const VariantEntry kVariants[]"):ker.index("#undef CTS_V")]]
     h = hashlib.sha256()

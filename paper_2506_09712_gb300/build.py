@@ -29,7 +29,7 @@ LIB_CHECKED = os.path.join(BUILD_CHECKED, "libcts_checked.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["cts_kernels.cu", "cts_runtime.cu", "cts_host.cpp", "cts_noalloc.cu"]
-HEADERS = ["cts_internal.h", "cts_host_impl.h"]
+HEADERS = ["cts_internal.h", "cts_host_impl.h", "cts_pairs.cuh"]
 
 
 def nvcc() -> str:

@@ -5,11 +5,12 @@
 // pool, a process with a fixed device-memory budget, code that must not
 // synchronise the device the way cudaMalloc/cudaFree can).  For them,
 // cts_field_noalloc computes the same pair field as the library's field
-// kernel, with the caller's device buffers for inputs and output, and keeps
-// its working storage (per-carrier FP64 accumulators and per-tile counters)
-// in one file-scope __device__ array of fixed size instead of allocating it.
-// That array is part of the library image: every GPU that loads the library
-// holds it (about 3 MB) until the process exits.
+// kernel, with the caller's device buffers for inputs and output.  Inputs of up
+// to kNaDirect carriers need no working storage; larger ones evaluate each
+// unordered pair once and keep per-carrier FP64 accumulators in one file-scope
+// __device__ array of fixed size instead of allocating it.  That array is part
+// of the library image: every GPU that loads the library holds it (about 3 MB)
+// until the process exits.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -17,127 +18,242 @@
 #include <mutex>
 
 #include "cts.h"
+#include "cts_pairs.cuh"
 
 namespace {
 
+using namespace cts;
+
 constexpr int kNaMaxCarriers = 131072;  // largest n_h + n_e accepted
-constexpr int kNaThreads = 128;
-constexpr int kNaR = 4;                 // carriers per thread
-constexpr int kNaTile = kNaThreads * kNaR;
-constexpr int kNaMaxTiles = kNaMaxCarriers / kNaTile;
-constexpr int kNaStage = 256;           // sources staged in shared memory per pass
-constexpr int kNaMaxSplit = 32;
 constexpr int kNaMaxDevices = 64;
-// layout: acc[3][kNaMaxCarriers] FP64, then one 64-bit counter per tile
-constexpr size_t kNaWords = 3 * (size_t)kNaMaxCarriers + kNaMaxTiles;
+// Up to here the direct kernel (one launch, every ordered pair), above the
+// symmetric one (a memset and two launches).
+constexpr int kNaDirect = 20000;
+// layout: the unit counter (word 0), then acc[3][n] FP64 from word kNaAcc
+constexpr int kNaAcc = 32;
+constexpr size_t kNaWords = kNaAcc + 3 * (size_t)kNaMaxCarriers;
 
 static __device__ __align__(256) unsigned long long cts_noalloc_scratch[kNaWords];
 
-__device__ __forceinline__ float na_rsqrt(float v) {
-  float r;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
-  return r;
-}
-
 // Eq. 4 read as a field: E_i = k sum_j s_j (r_i - r_j) / (|r_i - r_j|^2 + eps^2)^(3/2)
 // with s_j = +1 for the first n_h carriers (holes) and -1 for the rest.
-// Block b handles tile b / n_split of the i's against source range split
-// b % n_split; the block that completes a tile's last split writes the tile's
-// output and returns its accumulators and counter to zero.
-__global__ void __launch_bounds__(kNaThreads) field_noalloc_kernel(
-    const float* __restrict__ x, const float* __restrict__ y, const float* __restrict__ z,
-    int n_h, int n_e, int n_split, float kc, float eps2, float* __restrict__ out,
-    unsigned long long* scratch) {
-  __shared__ float4 sj[kNaStage];
-  __shared__ int s_last;
-  const int n = n_h + n_e;
-  const int tile = blockIdx.x / n_split, split = blockIdx.x % n_split;
-  const int i0 = tile * kNaTile;
-  const int j0 = (int)((long long)n * split / n_split);
-  const int j1 = (int)((long long)n * (split + 1) / n_split);
-  double* acc = reinterpret_cast<double*>(scratch);
-  unsigned long long* count = scratch + 3 * (size_t)kNaMaxCarriers;
+//
+// Direct: a warp takes a row of four i's against one of n_split shares of the
+// sources (iterations of 64: two per lane, read straight from the caller's
+// arrays, which the L1 cache holds), reduces its sums over the lanes, and the
+// CTA adds a row's shares in order.  No working storage, no other launch.
+// Small inputs are bound by latency (one pass of dependent loads, one
+// reduction), larger ones by the FP32 pipe.
+constexpr int kNaWarps = 8;
 
-  float xi[kNaR], yi[kNaR], zi[kNaR], sx[kNaR], sy[kNaR], sz[kNaR], cx[kNaR], cy[kNaR],
-      cz[kNaR];
-#pragma unroll
-  for (int r = 0; r < kNaR; ++r) {
-    const int i = i0 + r * kNaThreads + threadIdx.x;
-    xi[r] = i < n ? x[i] : 0.0f;
-    yi[r] = i < n ? y[i] : 0.0f;
-    zi[r] = i < n ? z[i] : 0.0f;
-    sx[r] = sy[r] = sz[r] = cx[r] = cy[r] = cz[r] = 0.0f;
+template <bool NEG>
+__device__ __forceinline__ void na_sources(const float* __restrict__ x, const float* __restrict__ y,
+                                           const float* __restrict__ z, int j0, int n, int it0,
+                                           int it1, int lane, const float2 (&x2)[kTeamR],
+                                           const float2 (&y2)[kTeamR], const float2 (&z2)[kTeamR],
+                                           float2 (&ax)[kTeamR], float2 (&ay)[kTeamR],
+                                           float2 (&az)[kTeamR], float2 eps2) {
+  const int full = min(it1, n >> 6);
+#pragma unroll 2
+  for (int it = it0; it < full; ++it) {
+    const int j = j0 + 64 * it + lane;
+    row_pairs<NEG>(make_float2(__ldg(x + j), __ldg(x + j + 32)),
+                   make_float2(__ldg(y + j), __ldg(y + j + 32)),
+                   make_float2(__ldg(z + j), __ldg(z + j + 32)), x2, y2, z2, ax, ay, az, eps2);
   }
-  for (int jb = j0; jb < j1; jb += kNaStage) {
-    const int m = min(kNaStage, j1 - jb);
-    for (int t = threadIdx.x; t < m; t += kNaThreads) {
-      const int j = jb + t;
-      sj[t] = make_float4(x[j], y[j], z[j], j < n_h ? 1.0f : -1.0f);
-    }
-    __syncthreads();
-    float tx[kNaR], ty[kNaR], tz[kNaR];
+  if (max(it0, full) < it1) {  // the last, partly filled iteration
+    const int a = 64 * full + lane, b = a + 32;
+    auto at = [&](const float* p, int j) { return j < n ? __ldg(p + j0 + j) : kParked; };
+    row_pairs<NEG>(make_float2(at(x, a), at(x, b)), make_float2(at(y, a), at(y, b)),
+                   make_float2(at(z, a), at(z, b)), x2, y2, z2, ax, ay, az, eps2);
+  }
+}
+
+__global__ void __launch_bounds__(32 * kNaWarps) field_rows_kernel(
+    const float* __restrict__ x, const float* __restrict__ y, const float* __restrict__ z,
+    int n_h, int n_e, int n_split, float kc, float eps2s, float* __restrict__ out) {
+  __shared__ float part[kNaWarps][3 * kTeamR];
+  const int n = n_h + n_e, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int per = kNaWarps / n_split;  // rows of this CTA
+  const int i0 = kTeamR * (blockIdx.x * per + warp / n_split), split = warp % n_split;
+  const int ih = (n_h + 63) >> 6, its = ih + ((n_e + 63) >> 6);
+  const int it0 = its * split / n_split, it1 = its * (split + 1) / n_split;
+  float2 x2[kTeamR], y2[kTeamR], z2[kTeamR], ax[kTeamR], ay[kTeamR], az[kTeamR];
 #pragma unroll
-    for (int r = 0; r < kNaR; ++r) tx[r] = ty[r] = tz[r] = 0.0f;
-    for (int t = 0; t < m; ++t) {
-      const float4 q = sj[t];
+  for (int r = 0; r < kTeamR; ++r) {
+    const int i = min(i0 + r, n - 1);
+    x2[r] = make_float2(x[i], x[i]);
+    y2[r] = make_float2(y[i], y[i]);
+    z2[r] = make_float2(z[i], z[i]);
+    ax[r] = ay[r] = az[r] = make_float2(0.0f, 0.0f);
+  }
+  const float2 eps2 = make_float2(eps2s, eps2s);
+  if (i0 < n) {
+    if (it0 < ih)
+      na_sources<false>(x, y, z, 0, n_h, it0, min(it1, ih), lane, x2, y2, z2, ax, ay, az, eps2);
+    if (it1 > ih)
+      na_sources<true>(x, y, z, n_h, n_e, max(it0, ih) - ih, it1 - ih, lane, x2, y2, z2, ax, ay, az,
+                       eps2);
+  }
+  float v[3 * kTeamR];
 #pragma unroll
-      for (int r = 0; r < kNaR; ++r) {
-        const float dx = xi[r] - q.x, dy = yi[r] - q.y, dz = zi[r] - q.z;
-        const float r2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, eps2)));
-        const float rs = na_rsqrt(r2);
-        const float w = q.w * ((rs * rs) * rs);
-        tx[r] = fmaf(dx, w, tx[r]);
-        ty[r] = fmaf(dy, w, ty[r]);
-        tz[r] = fmaf(dz, w, tz[r]);
+  for (int r = 0; r < kTeamR; ++r) {
+    v[3 * r] = ax[r].x + ax[r].y;
+    v[3 * r + 1] = ay[r].x + ay[r].y;
+    v[3 * r + 2] = az[r].x + az[r].y;
+  }
+  team_reduce(v, lane);
+  if ((lane & 7) == 0) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) part[warp][3 * (lane >> 3) + c] = v[c];
+  }
+  __syncthreads();
+  // thread t: component t mod 3 of the CTA's carrier t / 3
+  if (threadIdx.x < 3 * kTeamR * per) {
+    const int row = threadIdx.x / (3 * kTeamR), e = threadIdx.x % (3 * kTeamR);
+    const int i = kTeamR * (blockIdx.x * per + row) + e / 3;
+    float sum = 0.0f;
+    for (int s = 0; s < n_split; ++s) sum += part[row * n_split + s][e];
+    if (i < n) out[(size_t)(e % 3) * n + i] = kc * sum;
+  }
+}
+
+// Symmetric: units of kNaB I blocks (256 carriers of one species, eight per
+// lane) x kNaT J tiles (64 carriers of one species), one warp per unit, pulled
+// from a counter; the pair loop of the symmetric step kernel.  A block's sums
+// over the unit's tiles and a tile's over its blocks are FP32 (at most 256 and
+// 2 x 256 terms); they are added to the carriers' FP64 accumulators by atomics.
+// Bound: the FP32 pipe, 14 lane operations per unordered pair.
+constexpr int kNaSymWarps = 12;
+constexpr int kNaB = 2, kNaT = 8;
+constexpr int kNaWarpFloats = 3 * 64 + kNaT * 3 * kSymTile;
+constexpr int kNaSmem = kNaSymWarps * kNaWarpFloats * 4;
+
+__global__ void __launch_bounds__(32 * kNaSymWarps, 1) field_sym_kernel(
+    const float* __restrict__ x, const float* __restrict__ y, const float* __restrict__ z,
+    int n_h, int n_e, float eps2, unsigned long long* scratch) {
+  extern __shared__ __align__(16) float na_smem[];
+  const int n = n_h + n_e, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float2* sx = reinterpret_cast<float2*>(na_smem + warp * kNaWarpFloats);
+  float2* sy = sx + 32;
+  float2* sz = sy + 32;
+  float* jacc = na_smem + warp * kNaWarpFloats + 3 * 64;
+  double* acc = reinterpret_cast<double*>(scratch + kNaAcc);
+  // the units in order: hole blocks x hole tiles (from the block row's first
+  // tile on), hole blocks x electron tiles, electron blocks x electron tiles;
+  // `first` is the number of the current block row's first unit
+  int sec = 0, row = 0, first = 0;
+  auto tiles = [](int m) { return (m + kSymTile - 1) / kSymTile; };
+  auto rows_of = [&](int s) { return (tiles(s == 2 ? n_e : n_h) + kNaB * kSymTpb - 1) / (kNaB * kSymTpb); };
+  auto units_of = [&](int s, int q) {
+    const int t = tiles(s ? n_e : n_h) - (s == 1 ? 0 : q * kNaB * kSymTpb);
+    return (t + kNaT - 1) / kNaT;
+  };
+  for (;;) {
+    int u = 0;
+    if (lane == 0) u = atomicAdd(reinterpret_cast<int*>(scratch), 1);
+    u = __shfl_sync(0xffffffffu, u, 0);
+    while (sec < 3) {
+      if (row >= rows_of(sec)) {
+        ++sec;
+        row = 0;
+      } else if (u >= first + units_of(sec, row)) {
+        first += units_of(sec, row++);
+      } else {
+        break;
       }
     }
+    if (sec == 3) return;
+    const bool same = sec != 1;
+    const int ibase = sec == 2 ? n_h : 0, ni = sec == 2 ? n_e : n_h;
+    const int jbase = sec ? n_h : 0, nj = sec ? n_e : n_h;
+    const int nti = tiles(ni), ntj = tiles(nj);
+    const int g0 = (same ? row * kNaB * kSymTpb : 0) + (u - first) * kNaT;
+    const int g1 = min(ntj, g0 + kNaT);
+    for (int e = lane; e < (g1 - g0) * 3 * kSymTile; e += 32) jacc[e] = 0.0f;
+    for (int b = row * kNaB; b < (row + 1) * kNaB && b * kSymTpb < nti; ++b) {
+      const int bt0 = b * kSymTpb, vt = min(kSymTpb, nti - bt0);
+      const int ga = same ? max(g0, bt0) : g0;
+      if (ga >= g1) continue;
+      float2 xi[kSymRI], yi[kSymRI], zi[kSymRI], aix[kSymRI], aiy[kSymRI], aiz[kSymRI];
 #pragma unroll
-    for (int r = 0; r < kNaR; ++r) {  // Kahan fold of this pass
-      float u = tx[r] - cx[r], v = sx[r] + u;
-      cx[r] = (v - sx[r]) - u;
-      sx[r] = v;
-      u = ty[r] - cy[r];
-      v = sy[r] + u;
-      cy[r] = (v - sy[r]) - u;
-      sy[r] = v;
-      u = tz[r] - cz[r];
-      v = sz[r] + u;
-      cz[r] = (v - sz[r]) - u;
-      sz[r] = v;
-    }
-    __syncthreads();
-  }
+      for (int r = 0; r < kSymRI; ++r) {
+        const int ii = b * kSymBlock + r * 32 + lane;
+        const bool on = ii < ni;
+        const float px = on ? __ldg(x + ibase + ii) : kParked;
+        const float py = on ? __ldg(y + ibase + ii) : kParked;
+        const float pz = on ? __ldg(z + ibase + ii) : kParked;
+        xi[r] = make_float2(px, px);
+        yi[r] = make_float2(py, py);
+        zi[r] = make_float2(pz, pz);
+        aix[r] = aiy[r] = aiz[r] = make_float2(0.0f, 0.0f);
+      }
+      // a tile's positions, fetched one tile ahead
+      float2 px, py, pz;
+      auto fetch = [&](int g) {
+        const int a = g * kSymTile + lane, c = a + 32;
+        auto at = [&](const float* p, int j) { return j < nj ? __ldg(p + jbase + j) : kParked; };
+        px = make_float2(at(x, a), at(x, c));
+        py = make_float2(at(y, a), at(y, c));
+        pz = make_float2(at(z, a), at(z, c));
+      };
+      fetch(ga);
+      for (int g = ga; g < g1; ++g) {
+        __syncwarp();
+        sx[lane] = px;
+        sy[lane] = py;
+        sz[lane] = pz;
+        __syncwarp();
+        if (g + 1 < g1) fetch(g + 1);
+        float2 ajx = make_float2(0.0f, 0.0f), ajy = ajx, ajz = ajx;
+        const int qd = same ? min(g - bt0, kSymTpb) : kSymTpb;
+        if (vt == kSymTpb && qd == kSymTpb)
+          sym_tile_pairs<kSymRI, kSymTpb, 2>(sx, sy, sz, lane, xi, yi, zi, aix, aiy, aiz, ajx, ajy,
+                                             ajz, eps2, qd, vt);
+        else
+          sym_tile_pairs<kSymRI, -1, 1>(sx, sy, sz, lane, xi, yi, zi, aix, aiy, aiz, ajx, ajy, ajz,
+                                        eps2, qd, vt);
+        float* jt = jacc + (g - g0) * 3 * kSymTile;
+        jt[lane] += ajx.x;
+        jt[32 + lane] += ajx.y;
+        jt[kSymTile + lane] += ajy.x;
+        jt[kSymTile + 32 + lane] += ajy.y;
+        jt[2 * kSymTile + lane] += ajz.x;
+        jt[2 * kSymTile + 32 + lane] += ajz.y;
+      }
+      const double sj = sec ? -1.0 : 1.0;  // the J species' sign
 #pragma unroll
-  for (int r = 0; r < kNaR; ++r) {
-    const int i = i0 + r * kNaThreads + threadIdx.x;
-    if (i < n) {
-      atomicAdd(acc + i, (double)sx[r] - (double)cx[r]);
-      atomicAdd(acc + kNaMaxCarriers + i, (double)sy[r] - (double)cy[r]);
-      atomicAdd(acc + 2 * kNaMaxCarriers + i, (double)sz[r] - (double)cz[r]);
+      for (int r = 0; r < kSymRI; ++r) {
+        const int ii = b * kSymBlock + r * 32 + lane;
+        if (ii < ni) {
+          double* a = acc + ibase + ii;
+          atomicAdd(a, sj * (double)(aix[r].x + aix[r].y));
+          atomicAdd(a + n, sj * (double)(aiy[r].x + aiy[r].y));
+          atomicAdd(a + 2 * (size_t)n, sj * (double)(aiz[r].x + aiz[r].y));
+        }
+      }
     }
-  }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const unsigned long long old = atomicAdd(count + tile, 1ull);
-    s_last = old == (unsigned long long)(n_split - 1);
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-#pragma unroll
-  for (int r = 0; r < kNaR; ++r) {
-    const int i = i0 + r * kNaThreads + threadIdx.x;
-    if (i < n) {
-      out[i] = kc * (float)__ldcg(acc + i);
-      out[n + i] = kc * (float)__ldcg(acc + kNaMaxCarriers + i);
-      out[2 * n + i] = kc * (float)__ldcg(acc + 2 * kNaMaxCarriers + i);
-      acc[i] = 0.0;
-      acc[kNaMaxCarriers + i] = 0.0;
-      acc[2 * kNaMaxCarriers + i] = 0.0;
+    __syncwarp();
+    const double si = sec == 2 ? 1.0 : -1.0;  // minus the I species' sign
+    for (int e = lane; e < (g1 - g0) * kSymTile; e += 32) {
+      const int t = e / kSymTile, j = (g0 + t) * kSymTile + e % kSymTile;
+      if (j < nj) {
+        const float* src = jacc + t * 3 * kSymTile + e % kSymTile;
+        double* a = acc + jbase + j;
+        atomicAdd(a, si * (double)src[0]);
+        atomicAdd(a + n, si * (double)src[kSymTile]);
+        atomicAdd(a + 2 * (size_t)n, si * (double)src[2 * kSymTile]);
+      }
     }
+    __syncwarp();
   }
-  if (threadIdx.x == 0) count[tile] = 0ull;
+}
+
+__global__ void __launch_bounds__(256) field_out_kernel(const unsigned long long* scratch, int n3,
+                                                        float kc, float* __restrict__ out) {
+  const double* acc = reinterpret_cast<const double*>(scratch + kNaAcc);
+  const int e = blockIdx.x * 256 + threadIdx.x;
+  if (e < n3) out[e] = kc * (float)acc[e];
 }
 
 // Device address of the scratch array, looked up once per device (with that
@@ -155,6 +271,9 @@ int na_setup(int dev, void** addr, int* sms) {
     if (prop.major != 10 || prop.minor != 3) return SIM_ENODEV;
     void* p = nullptr;
     if (cudaGetSymbolAddress(&p, cts_noalloc_scratch) != cudaSuccess || !p) return SIM_ECUDA;
+    if (cudaFuncSetAttribute(field_sym_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kNaSmem) != cudaSuccess)
+      return SIM_ECUDA;
     g_na_addr[dev] = p;
     g_na_sms[dev] = prop.multiProcessorCount;
   }
@@ -182,24 +301,26 @@ extern "C" int cts_field_noalloc(const float* dev_x, const float* dev_y, const f
   const int rc = na_setup(dev, &scratch, &sms);
   if (rc != SIM_OK) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  const int tiles = (int)((n + kNaTile - 1) / kNaTile);
-  // the accumulators and counters this call uses start at zero
-  double* acc = (double*)scratch;
-  for (int c = 0; c < 3; ++c)
-    if (cudaMemsetAsync(acc + (size_t)c * kNaMaxCarriers, 0, (size_t)n * sizeof(double), s) !=
-        cudaSuccess)
-      return SIM_ECUDA;
-  if (cudaMemsetAsync((unsigned long long*)scratch + 3 * (size_t)kNaMaxCarriers, 0,
-                      (size_t)tiles * sizeof(unsigned long long), s) != cudaSuccess)
-    return SIM_ECUDA;
-  int n_split = (4 * sms + tiles - 1) / tiles;
-  n_split = n_split < 1 ? 1 : (n_split > kNaMaxSplit ? kNaMaxSplit : n_split);
-  if (n_split > n / 64) n_split = (int)(n / 64 > 1 ? n / 64 : 1);
   const double e = 1.602176634e-19, eps0 = 8.8541878128e-12;
   const float kc = (float)(e / (4.0 * M_PI * eps0 * eps_r) * 1e6);
   const double eps = softening_um > 0 ? softening_um : 1e-6;
-  field_noalloc_kernel<<<tiles * n_split, kNaThreads, 0, s>>>(
-      dev_x, dev_y, dev_z, n_h, n_e, n_split, kc, (float)(eps * eps), dev_E,
-      (unsigned long long*)scratch);
+  const float eps2 = (float)(eps * eps);
+  if (n <= kNaDirect) {
+    // shares of a row's sources: as many as keep about 32 warps per SM busy
+    const int rows = (int)((n + kTeamR - 1) / kTeamR);
+    int split = 1;
+    while (split < kNaWarps && (int64_t)rows * split < 32 * (int64_t)sms) split *= 2;
+    const int per = kNaWarps / split;
+    field_rows_kernel<<<(rows + per - 1) / per, 32 * kNaWarps, 0, s>>>(
+        dev_x, dev_y, dev_z, n_h, n_e, split, kc, eps2, dev_E);
+    return cudaGetLastError() == cudaSuccess ? SIM_OK : SIM_ECUDA;
+  }
+  // the counter and the accumulators this call uses start at zero
+  if (cudaMemsetAsync(scratch, 0, (kNaAcc + 3 * (size_t)n) * sizeof(double), s) != cudaSuccess)
+    return SIM_ECUDA;
+  unsigned long long* sc = (unsigned long long*)scratch;
+  field_sym_kernel<<<sms, 32 * kNaSymWarps, kNaSmem, s>>>(dev_x, dev_y, dev_z, n_h, n_e, eps2, sc);
+  if (cudaGetLastError() != cudaSuccess) return SIM_ECUDA;
+  field_out_kernel<<<(int)((3 * n + 255) / 256), 256, 0, s>>>(sc, (int)(3 * n), kc, dev_E);
   return cudaGetLastError() == cudaSuccess ? SIM_OK : SIM_ECUDA;
 }

@@ -1,0 +1,147 @@
+// cts_pairs.cuh -- the pair loops of Eq. 4 shared by the step kernels
+// (cts_kernels.cu) and the allocation-free field (cts_noalloc.cu).  All work on
+// packed FP32 pairs (two-wide FMA), with one approximate rsqrt per pair.
+#pragma once
+#include <cuda_runtime.h>
+
+#include "cts_internal.h"
+
+namespace cts {
+
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// ---- each unordered pair once (the symmetric kernel's loop) ----------------
+// The pairs of one (block, tile) combination.  QD = kSymTpb: every i-slot
+// pairs with the tile both ways.  Otherwise tile t = r / 2 of the block pairs
+// both ways if t < qd, with itself (i sums only: every ordered pair of the
+// tile once) if t == qd, not at all if t > qd or t >= vt (tiles past the
+// species' end); QD in [0, kSymTpb) fixes qd at compile time (a full block's
+// own tiles), QD = -1 takes qd and vt at run time.  UNR rotation steps per
+// loop iteration.
+template <int RI, int QD, int UNR>
+__device__ __forceinline__ void sym_tile_pairs(const float2* __restrict__ sx,
+                                               const float2* __restrict__ sy,
+                                               const float2* __restrict__ sz, int lane,
+                                               const float2 (&xi)[RI], const float2 (&yi)[RI],
+                                               const float2 (&zi)[RI], float2 (&aix)[RI],
+                                               float2 (&aiy)[RI], float2 (&aiz)[RI], float2& ajx,
+                                               float2& ajy, float2& ajz, float eps2s, int qd_rt,
+                                               int vt_rt) {
+  const float2 m1 = make_float2(-1.0f, -1.0f);
+  const float2 eps2 = make_float2(eps2s, eps2s);
+  const int src = (lane + 1) & 31;
+  const int qd = QD >= 0 ? QD : qd_rt;
+  const int vt = QD >= 0 ? kSymTpb : vt_rt;
+#pragma unroll UNR
+  for (int s = 0; s < 32; ++s) {
+    const int jj = (lane + s) & 31;
+    const float2 xj = sx[jj], yj = sy[jj], zj = sz[jj];
+#pragma unroll
+    for (int r = 0; r < RI; ++r) {
+      const int t = r >> 1;
+      if (t >= vt || t > qd) continue;
+      const float2 dx = __ffma2_rn(xj, m1, xi[r]);
+      const float2 dy = __ffma2_rn(yj, m1, yi[r]);
+      const float2 dz = __ffma2_rn(zj, m1, zi[r]);
+      float2 r2 = __ffma2_rn(dz, dz, eps2);
+      r2 = __ffma2_rn(dy, dy, r2);
+      r2 = __ffma2_rn(dx, dx, r2);
+      const float2 rs = make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+      const float2 w = __fmul2_rn(__fmul2_rn(rs, rs), rs);
+      aix[r] = __ffma2_rn(dx, w, aix[r]);
+      aiy[r] = __ffma2_rn(dy, w, aiy[r]);
+      aiz[r] = __ffma2_rn(dz, w, aiz[r]);
+      if (t < qd) {
+        ajx = __ffma2_rn(dx, w, ajx);
+        ajy = __ffma2_rn(dy, w, ajy);
+        ajz = __ffma2_rn(dz, w, ajz);
+      }
+    }
+    ajx.x = __shfl_sync(0xffffffffu, ajx.x, src);
+    ajx.y = __shfl_sync(0xffffffffu, ajx.y, src);
+    ajy.x = __shfl_sync(0xffffffffu, ajy.x, src);
+    ajy.y = __shfl_sync(0xffffffffu, ajy.y, src);
+    ajz.x = __shfl_sync(0xffffffffu, ajz.x, src);
+    ajz.y = __shfl_sync(0xffffffffu, ajz.y, src);
+  }
+}
+
+// ---- every ordered pair, rows of four i's against sources over the lanes ---
+constexpr int kTeamR = 4;  // i's per row
+
+// acc_r += d w for two sources (the halves of qx, qy, qz), d = r_i - r_j, or
+// r_j - r_i (NEG); the i's positions duplicated.
+template <bool NEG>
+__device__ __forceinline__ void row_pairs(float2 qx, float2 qy, float2 qz,
+                                          const float2 (&x2)[kTeamR], const float2 (&y2)[kTeamR],
+                                          const float2 (&z2)[kTeamR], float2 (&ax)[kTeamR],
+                                          float2 (&ay)[kTeamR], float2 (&az)[kTeamR], float2 eps2) {
+  const float2 m1 = make_float2(-1.0f, -1.0f);
+#pragma unroll
+  for (int r = 0; r < kTeamR; ++r) {
+    const float2 dx = NEG ? __ffma2_rn(x2[r], m1, qx) : __ffma2_rn(qx, m1, x2[r]);
+    const float2 dy = NEG ? __ffma2_rn(y2[r], m1, qy) : __ffma2_rn(qy, m1, y2[r]);
+    const float2 dz = NEG ? __ffma2_rn(z2[r], m1, qz) : __ffma2_rn(qz, m1, z2[r]);
+    float2 r2 = __ffma2_rn(dz, dz, eps2);
+    r2 = __ffma2_rn(dy, dy, r2);
+    r2 = __ffma2_rn(dx, dx, r2);
+    const float2 rs = make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+    const float2 w = __fmul2_rn(__fmul2_rn(rs, rs), rs);
+    ax[r] = __ffma2_rn(dx, w, ax[r]);
+    ay[r] = __ffma2_rn(dy, w, ay[r]);
+    az[r] = __ffma2_rn(dz, w, az[r]);
+  }
+}
+
+// acc_r += d w over iterations [it0, it1) of 64 sources from x[], y[], z[]
+// (float2 per lane and iteration), d = r_i - r_j, or r_j - r_i (NEG).
+template <bool NEG>
+__device__ __forceinline__ void team_pairs(const float* __restrict__ xs,
+                                           const float* __restrict__ ys,
+                                           const float* __restrict__ zs, int lane, int it0,
+                                           int it1, const float (&xi)[kTeamR],
+                                           const float (&yi)[kTeamR], const float (&zi)[kTeamR],
+                                           float2 (&ax)[kTeamR], float2 (&ay)[kTeamR],
+                                           float2 (&az)[kTeamR], float eps2s) {
+  const float2 eps2 = make_float2(eps2s, eps2s);
+  float2 x2[kTeamR], y2[kTeamR], z2[kTeamR];
+#pragma unroll
+  for (int r = 0; r < kTeamR; ++r) {
+    x2[r] = make_float2(xi[r], xi[r]);
+    y2[r] = make_float2(yi[r], yi[r]);
+    z2[r] = make_float2(zi[r], zi[r]);
+  }
+#pragma unroll 2
+  for (int it = it0; it < it1; ++it) {
+    const int j = 64 * it + 2 * lane;
+    row_pairs<NEG>(*reinterpret_cast<const float2*>(xs + j), *reinterpret_cast<const float2*>(ys + j),
+                   *reinterpret_cast<const float2*>(zs + j), x2, y2, z2, ax, ay, az, eps2);
+  }
+}
+
+// Sums the four rows' three components over the warp's lanes (a fixed tree);
+// lane l with l mod 8 == 0 ends with carrier l / 8's sums in v[0..2].
+__device__ __forceinline__ void team_reduce(float (&v)[3 * kTeamR], int lane) {
+  static_assert(kTeamR == 4, "two halving exchanges");
+  const bool h16 = lane & 16, h8 = lane & 8;
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    const float give = h16 ? v[q] : v[q + 6], keep = h16 ? v[q + 6] : v[q];
+    v[q] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const float give = h8 ? v[q] : v[q + 3], keep = h8 ? v[q + 3] : v[q];
+    v[q] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+  }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+    for (int q = 0; q < 3; ++q) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+}
+
+}  // namespace cts
