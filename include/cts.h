@@ -121,7 +121,8 @@ typedef struct sim_options_t {
   int32_t mode;            /* CTS_MODE_* */
   int32_t device;          /* CUDA device ordinal */
   int32_t max_slots;       /* events resident at once (default 256) */
-  int32_t chunk_steps;     /* steps per chunk between host checks (default 32) */
+  int32_t chunk_steps;     /* steps per chunk between host checks (default 32; up
+                              to 128 while only a little work runs) */
   int64_t max_carriers;    /* carrier arena capacity (default: from budget) */
   int64_t hbm_budget_bytes;/* device bytes the handle may allocate (default 1 GiB) */
   int32_t queue_capacity;  /* bound of the admission queue (default 65536) */

@@ -98,6 +98,13 @@ constexpr int kSymVariantPlain = 0;  // sym_nt384_r8_warp
 // carriers: 38.7 -> 92.1 us a step with them, the team kernel 40.3 -> 50.4).
 constexpr double kTeamMaxLoad = 2.4e4;
 constexpr double kTeamMaxLoadPixels = 4.8e4;
+// Steps of a team kernel's chunk when the caller leaves chunk_steps to the
+// library: a chunk's host round (plan, launches, copies, one synchronisation)
+// takes about 40 us, as long as eight steps of a small event, while a longer
+// chunk only delays the compaction of collected carriers and the next
+// admission.  One 3 keV photon (111 steps): four chunks of 32 723 us, one of
+// 128 637 us.  Pixel signals keep 32 (their record is copied per chunk).
+int team_steps(double W) { return W < 2.0e7 ? 128 : W < 6.0e7 ? 64 : kDefaultK; }
 // a team's CTAs have at least this many rows of kTeamRow carriers each (the
 // step of an 829-carrier event no longer shortens beyond 52 CTAs)
 constexpr int kTeamMinRows = 4;
@@ -236,6 +243,7 @@ struct sim_t {
   TeamEntry* d_team = nullptr;  // the team kernel's CTAs [sm_count]
   TeamEntry* h_team = nullptr;
   int team_grid = 0;        // CTAs of the current chunk (0: another kernel runs)
+  int chunk_K = 1;          // steps of the last chunk
   size_t team_smem = 0;     // their dynamic shared memory
 
   // host state
@@ -954,7 +962,7 @@ int set_variant(sim_t* s, int v);
 int run_chunk(sim_t* s) {
   NvtxRange range("cts chunk");
   const bool plain = s->opt.mode == CTS_MODE_PLAIN;
-  const int K = plain ? 1 : s->K;
+  int K = plain ? 1 : s->K;
   bool team = false;
   s->team_grid = 0;
   s->sym_level = 0;
@@ -1026,6 +1034,7 @@ int run_chunk(sim_t* s) {
         !s->opt.step_launches) {
       rcv = plan_team(s, &team);
       if (rcv) return rcv;
+      if (team && s->opt.chunk_steps == 0 && !s->d_induced_px) K = std::max(K, team_steps(W));
     }
   }
   // one launch for the whole chunk: the queue replays the step's pieces K
@@ -1050,6 +1059,7 @@ int run_chunk(sim_t* s) {
   if (rc) return rc;
   const int gi = 2 * s->variant + (multi ? 1 : 0);
   const int nl = (multi || sph || team) ? 1 : K;  // step-kernel launches in the chunk
+  s->chunk_K = K;
   CK(cudaEventRecord(s->ev0, s->stream));
   // (the grids of the team and the spherical kernel follow the running events:
   // they are launched directly)
@@ -1230,7 +1240,7 @@ int pump(sim_t* s, bool defer, bool* progressed) {
     }
     if (s->h_induced || s->h_induced_px) {
       // the steps this chunk executed for the slot, in order
-      const int K = s->opt.mode == CTS_MODE_PLAIN ? 1 : s->K;
+      const int K = s->chunk_K;
       const int64_t ran = std::min<int64_t>(std::max<int64_t>(m.n_steps - h.n_steps, 0), K);
       for (int64_t kk = 0; kk < ran; ++kk) {
         if (s->h_induced) {
