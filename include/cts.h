@@ -134,7 +134,7 @@ typedef struct sim_options_t {
                               (8 warps) below 2.6e8 pairs, up to 3072
                               carriers, and once an event has more than 640
                               tiles of 64 carriers -- the per-pair kernel
-                              (variant 2) below that, and below 2.4e4 times
+                              (variant 2) below that, and below 1.6e4 times
                               the largest event's carriers the team kernel (a
                               team of SMs per event; reported as variant 2); SERVE: variant 13 from
                               2.8e8 pairs, else variant 2; PLAIN: variant 1 */

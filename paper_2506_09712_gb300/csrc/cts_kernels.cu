@@ -404,27 +404,31 @@ __device__ __noinline__ void window_potentials(double x, double y, double z, dou
   for (int n = -M; n <= M; ++n) {
     const float zeta = fmaf((float)n, h2, zf);
     const float az = fabsf(zeta), sg = zeta < 0.0f ? -1.0f : 1.0f, z2 = zeta * zeta;
-    const bool far = uv < 0.1f * z2;
-    const float inv = 1.0f / zeta;
+    // corner (i, j) is the upper-right corner of pixel (i-1, j-1), the
+    // upper-left of (i, j-1), the lower-right of (i-1, j), the lower-left of (i, j)
+    auto add = [&](int i, int j, float f) {
+      if (i >= 1 && j >= 1) acc[(j - 1) * 3 + (i - 1)] += f;
+      if (i <= 2 && j >= 1) acc[(j - 1) * 3 + i] -= f;
+      if (i >= 1 && j <= 2) acc[j * 3 + (i - 1)] -= f;
+      if (i <= 2 && j <= 2) acc[j * 3 + i] += f;
+    };
+    if (uv < 0.1f * z2) {
+      const float inv = 1.0f / zeta;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+      for (int j = 0; j < 4; ++j)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float r2 = fmaf(u[i], u[i], fmaf(v[j], v[j], z2));
-        float f;
-        if (far) {
-          const float t = u[i] * v[j] * inv * rsqrtf(r2), t2 = t * t;
-          f = t * fmaf(t2, fmaf(t2, fmaf(t2, -1.0f / 7.0f, 0.2f), -1.0f / 3.0f), 1.0f);
-        } else {
-          f = sg * atan2f(u[i] * v[j], az * sqrtf(r2));
+        for (int i = 0; i < 4; ++i) {
+          const float t =
+              u[i] * v[j] * inv * rsqrtf(fmaf(u[i], u[i], fmaf(v[j], v[j], z2))), t2 = t * t;
+          add(i, j, t * fmaf(t2, fmaf(t2, fmaf(t2, -1.0f / 7.0f, 0.2f), -1.0f / 3.0f), 1.0f));
         }
-        // corner (i, j) is the upper-right corner of pixel (i-1, j-1), the
-        // upper-left of (i, j-1), the lower-right of (i-1, j), the lower-left of (i, j)
-        if (i >= 1 && j >= 1) acc[(j - 1) * 3 + (i - 1)] += f;
-        if (i <= 2 && j >= 1) acc[(j - 1) * 3 + i] -= f;
-        if (i >= 1 && j <= 2) acc[j * 3 + (i - 1)] -= f;
-        if (i <= 2 && j <= 2) acc[j * 3 + i] += f;
-      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          add(i, j, sg * atan2f(u[i] * v[j],
+                                az * sqrtf(fmaf(u[i], u[i], fmaf(v[j], v[j], z2)))));
     }
   }
   const float inv2pi = 0.159154943091895336f, q2 = pf * pf * (1.0f / 6.0f);

@@ -58,7 +58,7 @@ constexpr int64_t kDefaultBudget = 1ll << 30;
 // species of 4000, 4 events 101.5; 146.5; 82.1; 97.0, 10 events 198.9; 182.1;
 // 140.9; 134.1.
 constexpr double kSymMinWork = 1.6e8;
-constexpr double kSymShortWork = 2.6e8;
+constexpr double kSymShortWork = 2.7e8;
 constexpr double kSymFullWork = 5.5e8;
 constexpr int kSymFullEvents = 18;
 constexpr double kSymShortCarriers = 3072.0;
@@ -87,23 +87,20 @@ constexpr int kSymVariantPlain = 0;  // sym_nt384_r8_warp
 // 1 / 8 / 32 / 64 events 4.8 / 18.2, 7.2 / 18.7, 19.8 / 21.2, 35.4 / 30.1; 2210
 // carriers, 1 / 8 / 16 events 7.5 / 25.1, 24.0 / 28.8, 45.6 / 41.5; 5525
 // carriers, 1 / 2 / 4 / 8 events 19.7 / 51.0, 33.4 / 50.6, 59.5 / 58.3,
-// 111.5 / 96.4; 8000 carriers, 1 / 4 events 27.3 / 59.0, 83.5 / 96.2: the two
-// meet at 2.1e4 to 3.1e4.  SERVE keeps the queue kernels: a cooperative launch
+// 111.5 / 96.4; 8000 carriers, 1 / 4 events 27.3 / 59.0, 83.5 / 96.2; 3000
+// carriers, 8 events 40.3 / 38.7: the two meet at 2.1e4 to 3.1e4, and the line
+// lies where the team kernel wins for every size.  SERVE keeps the queue kernels: a cooperative launch
 // waits until all its SMs are free at once, which would put a stream of
 // requests behind whatever else its process runs on the GPU (and the events of
 // a stream are meant to overlap: alone, an 8 keV event of a served stream
 // takes 8.7 ms with teams, 26 ms without).
-// With pixel signals the line lies at twice as much: the potentials of a tile's
-// 512 carriers are one CTA's work in the per-pair kernel (eight events of 3000
-// carriers: 38.7 -> 92.1 us a step with them, the team kernel 40.3 -> 50.4).
-constexpr double kTeamMaxLoad = 2.4e4;
-constexpr double kTeamMaxLoadPixels = 4.8e4;
+constexpr double kTeamMaxLoad = 1.6e4;
 // Steps of a team kernel's chunk when the caller leaves chunk_steps to the
 // library: a chunk's host round (plan, launches, copies, one synchronisation)
 // takes about 40 us, as long as eight steps of a small event, while a longer
 // chunk only delays the compaction of collected carriers and the next
 // admission.  One 3 keV photon (111 steps): four chunks of 32 723 us, one of
-// 128 637 us.  Pixel signals keep 32 (their record is copied per chunk).
+// 128 637 us. 
 int team_steps(double W) { return W < 2.0e7 ? 128 : W < 6.0e7 ? 64 : kDefaultK; }
 // a team's CTAs have at least this many rows of kTeamRow carriers each (the
 // step of an 829-carrier event no longer shortens beyond 52 CTAs)
@@ -1030,11 +1027,11 @@ int run_chunk(sim_t* s) {
     }
     int rcv = set_variant(s, full ? sym_v : kPairVariant);
     if (rcv) return rcv;
-    if (!serve && W < (s->d_induced_px ? kTeamMaxLoadPixels : kTeamMaxLoad) * max_n && !full && !s->field.spherical &&
+    if (!serve && W < kTeamMaxLoad * max_n && !full && !s->field.spherical &&
         !s->opt.step_launches) {
       rcv = plan_team(s, &team);
       if (rcv) return rcv;
-      if (team && s->opt.chunk_steps == 0 && !s->d_induced_px) K = std::max(K, team_steps(W));
+      if (team && s->opt.chunk_steps == 0) K = std::max(K, team_steps(W));
     }
   }
   // one launch for the whole chunk: the queue replays the step's pieces K
