@@ -131,7 +131,7 @@ typedef struct sim_options_t {
                               events hold at least 1.6e8 carrier pairs (sum
                               of N^2; 4.0e8 if they are smaller than 1536
                               carriers) -- variant 1 (12 warps per SM), or 13
-                              (8 warps) below 2.6e8 pairs, up to 3072
+                              (8 warps) below 2.7e8 pairs, up to 3072
                               carriers, and once an event has more than 640
                               tiles of 64 carriers -- the per-pair kernel
                               (variant 2) below that, and below 1.6e4 times
@@ -423,9 +423,10 @@ typedef struct sim_cluster_t {
  * noisy pixel energies pixel_keV[n_events x grid_n^2] (NULL to skip), and
  * adds to spectrum[n_bins] (NULL if n_bins = 0) one count per on-grid pixel
  * of every accepted cluster, in bin floor((e - spec_lo_keV) / spec_bin_keV).
- * All buffers are the caller's host memory; the call allocates device memory
- * for the copies and synchronises.  Returns SIM_OK, SIM_EINVAL, SIM_ENODEV
- * or SIM_ECUDA. */
+ * All buffers are the caller's host memory; the call holds device memory for
+ * the copies and synchronises.  Up to four such buffers of at most 64 MiB are
+ * kept for later calls (sim_readout, sim_generate) until a handle on the
+ * device is destroyed.  Returns SIM_OK, SIM_EINVAL, SIM_ENODEV or SIM_ECUDA. */
 int sim_readout(const sim_readout_params_t* prm, const int32_t* counts, const uint64_t* seeds,
                 const uint64_t* event_ids, int32_t n_events, int32_t device, double* pixel_keV,
                 sim_cluster_t* clusters, int64_t* spectrum);
@@ -450,8 +451,8 @@ typedef struct sim_gen_event_t {
 /* Generate n_events events (host array) on GPU `device`: pixel counts into
  * pixels[n_events x grid_n^2] (row-major per event) and carriers that land
  * off the grid into outside[n_events] (NULL to skip), both host memory.
- * grid_n 1 .. 32, alpha > 0, beta in [0.3, 20], n_pairs >= 0.  Allocates
- * device memory for the copies and synchronises.  Returns SIM_OK,
+ * grid_n 1 .. 32, alpha > 0, beta in [0.3, 20], n_pairs >= 0.  Holds
+ * device memory like sim_readout and synchronises.  Returns SIM_OK,
  * SIM_EINVAL, SIM_ENODEV or SIM_ECUDA. */
 int sim_generate(const sim_gen_event_t* events, int32_t n_events, double pitch_um, int32_t grid_n,
                  int32_t device, int32_t* pixels, int64_t* outside);

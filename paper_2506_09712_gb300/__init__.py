@@ -455,16 +455,16 @@ def sim_readout(counts, seeds, event_ids, beam_keV, n_bins=0, device=0, want_pix
     ids = np.ascontiguousarray(event_ids, dtype=np.uint64)
     prm = sim_readout_params_t(grid_n=g, n_bins=int(n_bins), beam_keV=float(beam_keV),
                                **{k: float(v) for k, v in prm_d.items()})
-    cl = (sim_cluster_t * max(n_ev, 1))()
+    # sim_cluster_t rows: four int32, then e_cluster and e[9] (96 bytes)
+    cl = np.zeros((max(n_ev, 1), 12))
     spec = np.zeros(max(int(n_bins), 1), np.int64)
     pix = np.zeros((n_ev, g, g)) if want_pixels else None
     _check(load().sim_readout(C.byref(prm), _ptr(counts, C.c_int32), _ptr(seeds, C.c_uint64),
                               _ptr(ids, C.c_uint64), n_ev, int(device),
-                              _ptr(pix, C.c_double) if want_pixels else None, cl,
+                              _ptr(pix, C.c_double) if want_pixels else None,
+                              _ptr(cl, sim_cluster_t),
                               _ptr(spec, C.c_int64) if n_bins > 0 else None), "sim_readout")
-    raw = np.frombuffer(cl, dtype=np.uint8, count=96 * n_ev).reshape(n_ev, 96)
-    ints = raw[:, :16].copy().view(np.int32).reshape(n_ev, 4)
-    dbl = raw[:, 16:].copy().view(np.float64).reshape(n_ev, 10)
+    ints, dbl = cl.view(np.int32)[:n_ev, :4], cl[:n_ev, 2:]
     out = dict(cluster=dbl[:, 1:], e_cluster=dbl[:, 0], accepted=ints[:, 0], vetoed=ints[:, 1],
                cx=ints[:, 2], cy=ints[:, 3], spectrum=spec[:int(n_bins)])
     if want_pixels:

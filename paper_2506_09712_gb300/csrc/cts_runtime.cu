@@ -1373,12 +1373,116 @@ struct DeviceGuard {
 int check_device(int device, int* sms) {
   int n = 0;
   if (cudaGetDeviceCount(&n) != cudaSuccess || n <= device || device < 0) return SIM_ENODEV;
-  cudaDeviceProp p;
-  if (cudaGetDeviceProperties(&p, device) != cudaSuccess) return SIM_ENODEV;
-  if (p.major != 10 || p.minor != 3) return SIM_ENODEV;  // built for sm_103a only
-  *sms = p.multiProcessorCount;
+  int major = 0, minor = 0;
+  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, device) != cudaSuccess ||
+      cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
+    return SIM_ENODEV;
+  if (major != 10 || minor != 3) return SIM_ENODEV;  // built for sm_103a only
   return SIM_OK;
 }
+
+// Device memory and a stream for a stateless entry point (sim_generate,
+// sim_readout), kept between calls: allocating and freeing them cost each call
+// about 0.2 ms, more than the kernels of a small one.  A call owns its
+// workspace while it runs, so calls from several threads each take their own.
+// At most kIdle workspaces of at most kIdleBytes stay behind; they are given
+// back when a handle on the device is destroyed, or when an allocation here
+// fails.
+struct Workspace {
+  int device = -1;
+  cudaStream_t stream = nullptr;
+  char* mem = nullptr;
+  size_t bytes = 0, used = 0;
+  // a piece of the buffer (256-byte aligned)
+  template <typename T>
+  T* take(size_t n) {
+    T* p = reinterpret_cast<T*>(mem + used);
+    used += (n * sizeof(T) + 255) / 256 * 256;
+    return p;
+  }
+};
+class WorkspacePool {
+ public:
+  static constexpr size_t kIdle = 4, kIdleBytes = size_t(64) << 20;
+  // `device` is current.  A workspace of at least `bytes`.
+  cudaError_t acquire(int device, size_t bytes, Workspace* out) {
+    {
+      std::lock_guard<std::mutex> lk(mu_);
+      for (size_t q = idle_.size(); q-- > 0;)
+        if (idle_[q].device == device) {
+          *out = idle_[q];
+          idle_.erase(idle_.begin() + (ptrdiff_t)q);
+          break;
+        }
+    }
+    if (out->mem) {
+      // memory of a context that was reset meanwhile is gone: forget it
+      cudaPointerAttributes at{};
+      if (cudaPointerGetAttributes(&at, out->mem) != cudaSuccess ||
+          at.type != cudaMemoryTypeDevice || at.device != device) {
+        cudaGetLastError();
+        *out = Workspace{};
+      }
+    }
+    out->device = device;
+    out->used = 0;
+    cudaError_t e = cudaSuccess;
+    if (!out->stream && (e = cudaStreamCreateWithFlags(&out->stream, cudaStreamNonBlocking)))
+      return e;
+    if (out->bytes < bytes) {
+      if (out->mem) cudaFree(out->mem);
+      out->mem = nullptr;
+      out->bytes = 0;
+      e = cudaMalloc((void**)&out->mem, bytes);
+      if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        trim(device);
+        e = cudaMalloc((void**)&out->mem, bytes);
+      }
+      if (e) return e;
+      out->bytes = bytes;
+    }
+    return cudaSuccess;
+  }
+  // Back after a call; `keep` is false when the call failed.
+  void release(const Workspace& w, bool keep) {
+    if (keep && w.bytes <= kIdleBytes) {
+      std::lock_guard<std::mutex> lk(mu_);
+      if (idle_.size() < kIdle) {
+        idle_.push_back(w);
+        return;
+      }
+    }
+    drop(w);
+  }
+  void trim(int device) {
+    std::vector<Workspace> out;
+    {
+      std::lock_guard<std::mutex> lk(mu_);
+      for (size_t q = idle_.size(); q-- > 0;)
+        if (idle_[q].device == device) {
+          out.push_back(idle_[q]);
+          idle_.erase(idle_.begin() + (ptrdiff_t)q);
+        }
+    }
+    for (const Workspace& w : out) drop(w);
+  }
+
+ private:
+  static void drop(const Workspace& w) {
+    if (w.mem) cudaFree(w.mem);
+    if (w.stream) cudaStreamDestroy(w.stream);
+  }
+  std::mutex mu_;
+  std::vector<Workspace> idle_;
+};
+// never destroyed: the driver may be gone when static objects are
+WorkspacePool& workspaces() {
+  static WorkspacePool* pool = new WorkspacePool;
+  return *pool;
+}
+size_t padded(size_t bytes) { return (bytes + 255) / 256 * 256; }
 
 int alloc_all(sim_t* s) {
   const int64_t C = s->capacity;
@@ -1647,6 +1751,7 @@ int sim_destroy(sim_t* s) {
   }
   cudaSetDevice(s->device);
   if (s->stream) cudaStreamSynchronize(s->stream);
+  workspaces().trim(s->device);
   free_all(s);
   delete s;
   return SIM_OK;
@@ -2320,32 +2425,29 @@ int sim_generate(const sim_gen_event_t* events, int32_t n_events, double pitch_u
   DeviceGuard guard(device);
   if (n_events == 0) return SIM_OK;
   const size_t ne = (size_t)n_events, np = (size_t)grid_n * grid_n;
-  GenEvent* dev = nullptr;
-  int32_t* dp = nullptr;
-  unsigned long long* dout = nullptr;
-  cudaStream_t st = nullptr;
+  static_assert(sizeof(int64_t) == sizeof(unsigned long long), "count layout");
   cudaError_t e = cudaSuccess;
-  std::vector<unsigned long long> hout(outside ? ne : 0);
+  Workspace w;
   do {
-    if ((e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking))) break;
-    if ((e = cudaMalloc(&dev, ne * sizeof(GenEvent)))) break;
-    if ((e = cudaMalloc(&dp, ne * np * sizeof(int32_t)))) break;
-    if ((e = cudaMalloc(&dout, ne * sizeof(unsigned long long)))) break;
+    if ((e = workspaces().acquire(device, padded(ne * sizeof(GenEvent)) +
+                                              padded(ne * np * sizeof(int32_t)) +
+                                              padded(ne * sizeof(unsigned long long)), &w)))
+      break;
+    const cudaStream_t st = w.stream;
+    GenEvent* dev = w.take<GenEvent>(ne);
+    int32_t* dp = w.take<int32_t>(ne * np);
+    unsigned long long* dout = w.take<unsigned long long>(ne);
     if ((e = cudaMemcpyAsync(dev, events, ne * sizeof(GenEvent), cudaMemcpyHostToDevice, st)))
       break;
     if ((e = launch_generate(dev, n_events, pitch_um, grid_n, dp, dout, st))) break;
     if ((e = cudaMemcpyAsync(pixels, dp, ne * np * sizeof(int32_t), cudaMemcpyDeviceToHost, st)))
       break;
-    if (outside && (e = cudaMemcpyAsync(hout.data(), dout, ne * sizeof(unsigned long long),
+    if (outside && (e = cudaMemcpyAsync(outside, dout, ne * sizeof(unsigned long long),
                                         cudaMemcpyDeviceToHost, st)))
       break;
-    if ((e = cudaStreamSynchronize(st))) break;
-    for (size_t k = 0; k < hout.size(); ++k) outside[k] = (int64_t)hout[k];
+    e = cudaStreamSynchronize(st);
   } while (0);
-  cudaFree(dev);
-  cudaFree(dp);
-  cudaFree(dout);
-  if (st) cudaStreamDestroy(st);
+  workspaces().release(w, e == cudaSuccess);
   return e == cudaSuccess ? SIM_OK : SIM_ECUDA;
 }
 
@@ -2375,25 +2477,25 @@ int sim_readout(const sim_readout_params_t* prm, const int32_t* counts, const ui
   r.veto_factor = prm->veto_factor;
   r.spec_lo_keV = prm->spec_lo_keV;
   r.spec_bin_keV = prm->spec_bin_keV;
-  int32_t* dc = nullptr;
-  unsigned long long *ds = nullptr, *di = nullptr, *dh = nullptr;
-  double* de = nullptr;
-  ClusterRec* dcl = nullptr;
-  cudaStream_t st = nullptr;
   cudaError_t e = cudaSuccess;
-  std::vector<unsigned long long> hist((size_t)std::max(prm->n_bins, 1), 0ull);
+  const size_t nb = (size_t)prm->n_bins;
+  std::vector<unsigned long long> hist(std::max<size_t>(nb, 1), 0ull);
+  Workspace w;
   do {
-    if ((e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking))) break;
-    if ((e = cudaMalloc(&dc, ne * np * sizeof(int32_t)))) break;
-    if ((e = cudaMalloc(&ds, ne * sizeof(unsigned long long)))) break;
-    if ((e = cudaMalloc(&di, ne * sizeof(unsigned long long)))) break;
-    if ((e = cudaMalloc(&dcl, ne * sizeof(ClusterRec)))) break;
-    if (pixel_keV && (e = cudaMalloc(&de, ne * np * sizeof(double)))) break;
-    if (prm->n_bins > 0) {
-      if ((e = cudaMalloc(&dh, (size_t)prm->n_bins * sizeof(unsigned long long)))) break;
-      if ((e = cudaMemsetAsync(dh, 0, (size_t)prm->n_bins * sizeof(unsigned long long), st)))
-        break;
-    }
+    if ((e = workspaces().acquire(
+             device, padded(ne * np * sizeof(int32_t)) + 2 * padded(ne * sizeof(uint64_t)) +
+                         padded(ne * sizeof(ClusterRec)) +
+                         padded(nb * sizeof(unsigned long long)) +
+                         (pixel_keV ? padded(ne * np * sizeof(double)) : 0), &w)))
+      break;
+    const cudaStream_t st = w.stream;
+    int32_t* dc = w.take<int32_t>(ne * np);
+    unsigned long long* ds = w.take<unsigned long long>(ne);
+    unsigned long long* di = w.take<unsigned long long>(ne);
+    ClusterRec* dcl = w.take<ClusterRec>(ne);
+    unsigned long long* dh = nb ? w.take<unsigned long long>(nb) : nullptr;
+    double* de = pixel_keV ? w.take<double>(ne * np) : nullptr;
+    if (dh && (e = cudaMemsetAsync(dh, 0, nb * sizeof(unsigned long long), st))) break;
     if ((e = cudaMemcpyAsync(dc, counts, ne * np * sizeof(int32_t), cudaMemcpyHostToDevice, st)))
       break;
     if ((e = cudaMemcpyAsync(ds, seeds, ne * sizeof(uint64_t), cudaMemcpyHostToDevice, st))) break;
@@ -2411,19 +2513,13 @@ int sim_readout(const sim_readout_params_t* prm, const int32_t* counts, const ui
     if (de && (e = cudaMemcpyAsync(pixel_keV, de, ne * np * sizeof(double),
                                    cudaMemcpyDeviceToHost, st)))
       break;
-    if (dh && (e = cudaMemcpyAsync(hist.data(), dh, (size_t)prm->n_bins * sizeof(unsigned long long),
+    if (dh && (e = cudaMemcpyAsync(hist.data(), dh, nb * sizeof(unsigned long long),
                                    cudaMemcpyDeviceToHost, st)))
       break;
     if ((e = cudaStreamSynchronize(st))) break;
-    for (int b = 0; b < prm->n_bins; ++b) spectrum[b] += (int64_t)hist[b];
+    for (size_t b = 0; b < nb; ++b) spectrum[b] += (int64_t)hist[b];
   } while (0);
-  cudaFree(dc);
-  cudaFree(ds);
-  cudaFree(di);
-  cudaFree(dcl);
-  if (de) cudaFree(de);
-  if (dh) cudaFree(dh);
-  if (st) cudaStreamDestroy(st);
+  workspaces().release(w, e == cudaSuccess);
   return e == cudaSuccess ? SIM_OK : SIM_ECUDA;
 }
 
