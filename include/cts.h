@@ -134,9 +134,10 @@ typedef struct sim_options_t {
                               (8 warps) below 2.7e8 pairs, up to 3072
                               carriers, and once an event has more than 640
                               tiles of 64 carriers -- the per-pair kernel
-                              (variant 2) below that, and below 1.6e4 times
-                              the largest event's carriers the team kernel (a
-                              team of SMs per event; reported as variant 2); SERVE: variant 13 from
+                              (variant 2) below that, and for few or small
+                              events (below 8.5e3 to 2.4e4 times the largest
+                              event's carriers) the team kernel (a team of
+                              SMs per event; reported as variant 2); SERVE: variant 13 from
                               2.8e8 pairs, else variant 2; PLAIN: variant 1 */
   int32_t disable_graphs;  /* 1 = launch K-step chunks directly, not as CUDA graphs */
   int32_t keep_final_xy;   /* 1 = keep collected (x, y) and retire steps for poll */

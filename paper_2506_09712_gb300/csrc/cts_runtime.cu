@@ -80,21 +80,31 @@ constexpr int kSymLargeTiles = 640;
 constexpr int kPairVariant = 1;  // nt256_r2_jpair_dyn
 constexpr int kSymVariantPlain = 0;  // sym_nt384_r8_warp
 // The team kernel takes a chunk while the running events' carrier pairs are
-// below kTeamMaxLoad times the largest event's carriers.  Below, a step is
-// bound by latency, which grows with the event in the per-pair kernel; above,
-// by the pair loop, where the per-pair kernel is the faster one (2.8e12 against
-// 2.2e12 pairs/s).  Microseconds per step, team / per-pair kernel: 829 carriers,
-// 1 / 8 / 32 / 64 events 4.8 / 18.2, 7.2 / 18.7, 19.8 / 21.2, 35.4 / 30.1; 2210
-// carriers, 1 / 8 / 16 events 7.5 / 25.1, 24.0 / 28.8, 45.6 / 41.5; 5525
-// carriers, 1 / 2 / 4 / 8 events 19.7 / 51.0, 33.4 / 50.6, 59.5 / 58.3,
-// 111.5 / 96.4; 8000 carriers, 1 / 4 events 27.3 / 59.0, 83.5 / 96.2; 3000
-// carriers, 8 events 40.3 / 38.7: the two meet at 2.1e4 to 3.1e4, and the line
-// lies where the team kernel wins for every size.  SERVE keeps the queue kernels: a cooperative launch
-// waits until all its SMs are free at once, which would put a stream of
-// requests behind whatever else its process runs on the GPU (and the events of
-// a stream are meant to overlap: alone, an 8 keV event of a served stream
-// takes 8.7 ms with teams, 26 ms without).
-constexpr double kTeamMaxLoad = 1.6e4;
+// below a line times the largest event's carriers (for equal events: their
+// number times their carriers).  Below, a step is bound by latency, which grows
+// with the event in the per-pair kernel; above, by the pair loop, where the
+// per-pair kernel is the faster one (2.8e12 against 2.2e12 pairs/s).
+// Microseconds per step, team / per-pair kernel: 829 carriers, 1 / 8 / 32 / 64
+// events 4.6 / 18.2, 7.0 / 18.7, 19.8 / 21.2, 35.4 / 30.1; 2210 carriers, 1 / 4 /
+// 8 / 16 events 7.3 / 25.1, 14.8 / 26.8, 24.0 / 28.8, 45.6 / 41.5; 5525 carriers,
+// 1 / 2 / 4 / 8 events 19.6 / 51.0, 33.4 / 50.6, 59.5 / 58.3, 111.5 / 96.4; 8000
+// carriers, 1 / 4 events 27.3 / 59.0, 83.5 / 96.2; 3000 carriers, 8 events 40.3 /
+// 38.7: the two meet at 2.1e4 (large events) to 2.6e4 (small ones).  Five or
+// more events of over kTeamSmallCarriers take it only up to kTeamMaxLoad: the
+// gain there is under a fifth, and the two kernels add the field in different
+// orders, which a few unstable close pairs amplify (5 to 17 keV clouds start
+// 0.1 um wide; their signals after 64 steps end 1e-6 to 1e-5 from a 64-bit run
+// in either kernel, by chance), so such batches keep the sums they had.
+// SERVE keeps the queue kernels: a cooperative launch waits until all its SMs
+// are free at once, which would put a stream of requests behind whatever else
+// its process runs on the GPU (and the events of a stream are meant to overlap:
+// alone, an 8 keV event of a served stream takes 8.7 ms with teams, 26 ms
+// without).
+constexpr int kTeamFewEvents = 4;
+constexpr int kTeamSmallCarriers = 1280;
+constexpr double kTeamMaxLoadFew = 2.1e4;    // up to kTeamFewEvents events
+constexpr double kTeamMaxLoadSmall = 2.4e4;  // events of up to kTeamSmallCarriers
+constexpr double kTeamMaxLoad = 8.5e3;
 // Steps of a team kernel's chunk when the caller leaves chunk_steps to the
 // library: a chunk's host round (plan, launches, copies, one synchronisation)
 // takes about 40 us, as long as eight steps of a small event, while a longer
@@ -1027,7 +1037,10 @@ int run_chunk(sim_t* s) {
     }
     int rcv = set_variant(s, full ? sym_v : kPairVariant);
     if (rcv) return rcv;
-    if (!serve && W < kTeamMaxLoad * max_n && !full && !s->field.spherical &&
+    const double team_load = n_run <= kTeamFewEvents         ? kTeamMaxLoadFew
+                             : max_n <= kTeamSmallCarriers ? kTeamMaxLoadSmall
+                                                           : kTeamMaxLoad;
+    if (!serve && W < team_load * max_n && !full && !s->field.spherical &&
         !s->opt.step_launches) {
       rcv = plan_team(s, &team);
       if (rcv) return rcv;
