@@ -656,7 +656,8 @@ def run_ours(args, rank, world, local):
                            l2="flushed (256 MiB write) before every timed step",
                            variant=args.variant or
                            "default: chosen per chunk, the symmetric kernel while the resident "
-                           "pair work fills the GPU, the per-pair kernel below",
+                           "pair work fills the GPU, the per-pair and the team "
+                           "kernel below",
                            variant_table=table),
             "events_per_s": events_per_s,
             "roofline": roof, "e2e": e2e, "clocks": clocks, "gpu_launches": launches,

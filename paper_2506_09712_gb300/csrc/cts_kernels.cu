@@ -7,8 +7,10 @@
 //                 then drift (Eq. 6), mobility, diffusion and the FP64
 //                 position update of Eqs. 3 and 5, collection and exit.
 //                 Persistent CTAs pull (event, i-tile, j-split) units from a
-//                 per-step counter; j-splits are combined in FP64 by the CTA
-//                 that finishes last.
+//                 per-step counter; j-splits are combined by the CTA that
+//                 finishes last.
+//   sym_kernel    the same with each unordered pair evaluated once.
+//   team_kernel   the same for few events: a team of CTAs per event.
 //   update_kernel the update alone (two-launch PLAIN path).
 //   init_kernel   the initial cloud of each new event (Algorithm 1, Eq. 2).
 //   close_kernel  end-of-chunk bookkeeping and order-preserving compaction.
